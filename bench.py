@@ -318,6 +318,22 @@ def run_ours(args):
                                   "k_weo_apply2 144 B (averaged: 264 B), links 2 x 288 B per site per application"
                                   + (", clover blocks 288 B per site per application (A_oo^{-1} on the odd "
                                      "sites, A_ee on the even ones)" if W.csw else ""))
+    if W.kind == "lap" and apply_launches == 0 and prof[3][1] > 0:
+        # the cluster-resident solver: one kernel does every solve on chip, so its roofline is the SMs'
+        # shared-memory bandwidth.  Bytes per inner iteration and half-lattice entry: p and e read and
+        # written (16), two hops of seven 16-byte quads and one word per four entries (58), t written and
+        # p read (8)
+        sms = torch.cuda.get_device_properties(local).multi_processor_count
+        b_it = 41.0
+        achieved = inner_iters * N * b_it / (prof[3][1] / 1e3) / 1e9
+        top = sms * 128.0 * (clocks.get("sm_mhz") or 2070.0) * 1e6 / 1e9
+        roofline = {"bound": "shared memory", "kernel": "k_lap_resident<float> (whole solve: sources, inner CG on the "
+                    "even Schur complement, FP64 outer steps, contraction)", "achieved": achieved, "peak": top,
+                    "unit": "GB/s", "frac": achieved / top, "peak_source": "%d SMs x 128 B x SM clock" % sms,
+                    "traffic": None, "traffic_source": "the inner iterations move no HBM bytes",
+                    "algorithmic_bytes_per_site_rhs": b_it, "launches": prof[3][0], "apply_ms_total": None,
+                    "apply_share_of_step": None, "kernel_ms_total": prof[3][1],
+                    "step_breakdown_ms": {"all_iterations": prof[3][1]}}
     if W.kind == "lap":
         n_vec, vec_sites = (6, N // 2) if eo else (5, N)
     else:

@@ -154,6 +154,13 @@ PT_API int pt_set_launch_limit(pt_ctx *ctx, int64_t n);
  *                a work item is cta_threads x sites_per_thread sites.  The
  *                Wilson kernels take one site per thread (pt_get_tuning
  *                reports 1).
+ * A Laplacian lattice that a thread-block cluster can hold on chip (up to
+ * 131,072 sites with even sides, 65,536 with odd ones, half of that in FP64) is solved by one
+ * kernel that keeps each right-hand side's vectors in shared memory and
+ * registers, unless group, graph_iters, overlap, cta_threads or
+ * sites_per_thread ask for a shape of the batched engine's work items other
+ * than the default, or a launch limit is set; pt_stats then counts one kernel
+ * launch, no graph launches and the resident right-hand sides.
  * seconds_per_rhs is an output of pt_autotune (device time per trial RHS). */
 typedef struct pt_tune {
     double delta;

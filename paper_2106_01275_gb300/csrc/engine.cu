@@ -15,24 +15,23 @@
 //
 // Every kernel walks a device-built list of (slot, site block) work items
 // with a grid sized to the GPU (persistent CTAs).  Per-slot reductions are
-// deterministic: each item writes its partial sum, and the last item of a
-// slot (atomic completion counter) sums the partials in a fixed order and
-// advances the slot's state machine.  The host only replays the graph and
-// reads one flag word per replay.
+// deterministic: each item writes its partial sum, and a finalize kernel sums
+// a slot's partials in a fixed order and advances its state machine.  The host
+// only replays the graph and reads one flag word per replay.
+//
+// Laplacian lattices that fit on chip take lap_resident.cu instead.
 #include <math.h>
 #include <stdio.h>
 #include <string.h>
 
 #include <vector>
 
-#include "pt_common.cuh"
+#include "engine.cuh"
 
 #define PT_BLOCK 256        // threads per engine work item
 
 enum { PH_EMPTY = 0, PH_START = 1, PH_OUTER = 2, PH_INNER = 3, PH_CONTRACT = 4, PH_DONE = 5 };
-enum { MODE_TRACE = 0, MODE_SOLVE = 1, MODE_GRAD = 2 };
 enum { LIST_CONTRACT = 0, LIST_OUTER = 1, LIST_INNER = 2 };
-enum { TASK_ADJ = 1 };      // source is P^T v (with g5 for Wilson)
 
 struct Slot {
     int task, phase, inner_it, total_it;
@@ -40,16 +39,6 @@ struct Slot {
     double bnorm2, rr, rr0, target2;
     double relres, pad3;
     Cx<double> alpha, beta, omega, rho;
-};
-
-struct Task {
-    int set, colour, comp, flags;
-    int cidx, pad0, pad1, pad2;   // cidx: which colouring (multi-colouring runs)
-};
-
-struct TaskStat {
-    int iters, outer;
-    double relres;
 };
 
 struct EP {
@@ -95,10 +84,6 @@ struct EP {
     double tol, delta;
     int maxit, max_inner;
 };
-
-#define FLAG_DONE 0
-#define FLAG_NUMERIC 1
-#define FLAG_NOCONV 2
 
 // ------------------------------------------------------------------ field access
 template <int KIND, typename S>
@@ -168,16 +153,6 @@ __device__ __forceinline__ Cx<double> source_val(const EP &P, const Task &tk, ui
         z = pt_noise(key, (uint64_t)src * dof + a, P.noise);
     }
     return Cx<double>{sg * z.re, sg * z.im};
-}
-
-// site index and coordinate along mu of x + p e_mu for 0 <= p < D_mu (the
-// engine reduces its displacements once on the host): an add and a
-// conditional subtract instead of a modulo
-__device__ __forceinline__ int shift_fwd(const Geom &g, int idx, const int x[4], int mu, int p, int *c_out) {
-    int c = x[mu] + p;
-    if (c >= g.D[mu]) c -= g.D[mu];
-    *c_out = c;
-    return idx + (c - x[mu]) * g.stride[mu];
 }
 
 // ------------------------------------------------------------------ work items and reductions
@@ -2573,30 +2548,6 @@ static void enqueue_iteration(const EngineRun &E, cudaStream_t st, const cudaEve
 static const int PROF_PAIRS_LAP[4][3] = {{0, 0, 1}, {1, 1, 2}, {2, 5, 6}, {3, 7, 8}};
 static const int PROF_PAIRS_WIL[6][3] = {{0, 0, 1}, {1, 1, 2}, {0, 2, 3}, {1, 3, 4}, {2, 5, 6}, {3, 7, 8}};
 
-struct EngineRequest {
-    int mode;
-    int n_tasks;
-    const Task *h_tasks;
-    const int32_t *col;
-    uint64_t seed;
-    int noise, mu, n_p, dilute, pshift;
-    const int *p_list;
-    const double *B_user;
-    double *X_user;
-    double tol;
-    int maxit;
-    int prec;
-    int R_force;               // >0: exact slot count (grad mode)
-    int n_lev = 0, n_pr = 0, m_fin = 0;   // nested trace mode (see EP)
-    const int32_t *lev_cols = nullptr;
-    const int *lev_anc = nullptr;
-    // outputs
-    std::vector<double> task_out;   // trace: [n_tasks][n_p] complex
-    std::vector<TaskStat> tstat;
-    double *x64_out;           // grad mode: device pointer to the solutions (valid until next call)
-    int R_used;
-};
-
 static size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 // the even-odd split needs every side even (each hop then joins opposite parities)
@@ -2630,6 +2581,17 @@ static pt_ctx::Tune engine_tuning(const pt_ctx *c, const pt_op *op, int prec) {
     return d;
 }
 
+// inner iterations of one cycle before the FP64 residual is formed anew
+static int engine_max_inner(int prec, int maxit) {
+    return prec == PT_PREC_FP64 ? maxit : prec == PT_PREC_MIXED_FP32 ? 4000 : 400;
+}
+
+// Laplacian: whether a tuning leaves the work items and graphs at their defaults
+static bool default_shape(const pt_ctx::Tune &t) {
+    return t.group == 1 && t.graph_iters == 8 && t.overlap == 0 && (t.cta_threads == 0 || t.cta_threads == PT_BLOCK) &&
+           (t.sites_per_thread == 0 || t.sites_per_thread == Tile<0>::SPT);
+}
+
 template <int KIND, typename S, typename LS>
 static int run_engine_t(const pt_op *op, EngineRequest &rq, pt_stats *stats) {
     pt_ctx *c = op->ctx;
@@ -2642,6 +2604,14 @@ static int run_engine_t(const pt_op *op, EngineRequest &rq, pt_stats *stats) {
     if (clv && !eo) {
         pt_set_error("the clover operator runs on the even-odd engine only (every side even; no gradient)");
         return PT_ERR_ARG;
+    }
+    if constexpr (KIND == 0) {
+        // a lattice that a thread-block cluster can hold is solved on chip, unless the
+        // caller's tuning shapes this engine's work items or graphs, or caps its launches
+        if (default_shape(tn) && c->launch_limit == 0 && pt_lap_resident_fits(op, rq, eo)) {
+            LapResidentPlan plan = {eo, tn.delta, cycle_slack(rq.prec), engine_max_inner(rq.prec, rq.maxit)};
+            return pt_lap_resident_run(op, rq, plan, stats);
+        }
     }
     const int nsite = eo ? g.N / 2 : g.N;
     const int64_t L = eo ? (int64_t)nsite * (KIND ? 24 : 1) : pt_field_reals(op);
@@ -2767,9 +2737,7 @@ static int run_engine_t(const pt_op *op, EngineRequest &rq, pt_stats *stats) {
     P.tol = rq.tol;
     P.maxit = rq.maxit;
     P.delta = tn.delta;
-    if (rq.prec == PT_PREC_FP64) P.max_inner = rq.maxit;
-    else if (rq.prec == PT_PREC_MIXED_FP32) P.max_inner = 4000;
-    else P.max_inner = 400;
+    P.max_inner = engine_max_inner(rq.prec, rq.maxit);
 
     cudaStream_t st = c->stream;
     PT_CUDA(cudaMemcpyAsync((void *)P.tasks, rq.h_tasks, (size_t)rq.n_tasks * sizeof(Task), cudaMemcpyHostToDevice, st));

@@ -1,0 +1,91 @@
+// Definitions shared by the batched solver engine (engine.cu) and the
+// cluster-resident Laplacian solver (lap_resident.cu).
+#pragma once
+
+#include <vector>
+
+#include "pt_common.cuh"
+
+enum { MODE_TRACE = 0, MODE_SOLVE = 1, MODE_GRAD = 2 };
+enum { TASK_ADJ = 1 };      // source is P^T v (with g5 for Wilson)
+
+struct Task {
+    int set, colour, comp, flags;
+    int cidx, pad0, pad1, pad2;   // cidx: which colouring (multi-colouring runs)
+};
+
+struct TaskStat {
+    int iters, outer;
+    double relres;
+};
+
+#define FLAG_DONE 0
+#define FLAG_NUMERIC 1
+#define FLAG_NOCONV 2
+#define FLAG_TIMEOUT 3
+
+struct EngineRequest {
+    int mode;
+    int n_tasks;
+    const Task *h_tasks;
+    const int32_t *col;
+    uint64_t seed;
+    int noise, mu, n_p, dilute, pshift;
+    const int *p_list;
+    const double *B_user;
+    double *X_user;
+    double tol;
+    int maxit;
+    int prec;
+    int R_force;               // >0: exact slot count (grad mode)
+    int n_lev = 0, n_pr = 0, m_fin = 0;   // nested trace mode (see EP)
+    const int32_t *lev_cols = nullptr;
+    const int *lev_anc = nullptr;
+    // outputs
+    std::vector<double> task_out;   // trace: [n_tasks][n_p] complex
+    std::vector<TaskStat> tstat;
+    double *x64_out;           // grad mode: device pointer to the solutions (valid until next call)
+    int R_used;
+};
+
+// site index and coordinate along mu of x + p e_mu for 0 <= p < D_mu (the
+// engine reduces its displacements once on the host): an add and a
+// conditional subtract instead of a modulo
+__device__ __forceinline__ int shift_fwd(const Geom &g, int idx, const int x[4], int mu, int p, int *c_out) {
+    int c = x[mu] + p;
+    if (c >= g.D[mu]) c -= g.D[mu];
+    *c_out = c;
+    return idx + (c - x[mu]) * g.stride[mu];
+}
+
+// |r|^2 at which an inner cycle that starts from the FP64 residual |r|^2 = rr
+// ends: a factor delta below its start, but the residual that the outer test
+// asks for (half of tol |b|) where that lies within `slack` (in |r|^2) of it.
+// Ending a little above the last target would buy one more FP64 residual and
+// one more restart for the few iterations between the two.
+__host__ __device__ __forceinline__ double cycle_target2(double delta, double slack, double tol, double b2, double rr) {
+    const double fin = 0.25 * tol * tol * b2, t = delta * delta * rr;
+    return t <= slack * fin ? fin : t;
+}
+// slack: FP32 storage carries a cycle a decade past the default delta of 1e-5
+// (the autotuner's usual choice is 1e-6); BF16 storage is at its limit at delta
+static inline double cycle_slack(int prec) { return prec == PT_PREC_MIXED_FP32 ? 100.0 : 4.0; }
+
+// CG keeps its search direction across an FP64 residual replacement (the
+// direction's weight is |r|^2 of the new residual over that of the last
+// iteration) as long as the new residual is the one the recursion had reached
+// (within half as much again); a fresh start would build up the Krylov space
+// anew at every cycle.
+#define PT_CG_KEEP 2.25
+
+// The inner tolerance and iteration bounds of a run, as run_engine_t sets them.
+struct LapResidentPlan {
+    bool eo;                   // even Schur complement (every side even) or the full system
+    double delta, slack;
+    int max_inner;
+};
+
+// Whether a Laplacian run fits the cluster-resident solver (lap_resident.cu).
+bool pt_lap_resident_fits(const pt_op *op, const EngineRequest &rq, bool eo);
+// Runs it: fills rq.task_out, rq.tstat and *stats as the engine does.
+int pt_lap_resident_run(const pt_op *op, EngineRequest &rq, const LapResidentPlan &plan, pt_stats *stats);
