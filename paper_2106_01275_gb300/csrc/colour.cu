@@ -4,12 +4,12 @@
 // The greedy walk is sequential by definition (Sec. 4: the visit of each node
 // depends on the colours of the nodes visited before it), so one CTA walks the
 // visit order.  What is parallel is the gather of the neighbourhood's colours
-// (Sec. 4 notes it is read-only): the CTA's threads split the stencil, stamp
-// the colours they see into a shared-memory table, and search it for the
-// first free colour.  Lattices whose 16-bit colours fit in shared memory keep
-// them there (k_colour_walk); larger ones keep them in an extended array in
-// global memory, read through L1, with two nodes in flight per barrier
-// (k_colour_walk_ext).
+// (Sec. 4 notes it is read-only): k_colour_window gathers for 31 nodes at once
+// while one warp settles the 31 before them in order.  Stencils whose stamps
+// do not fit 31 times in shared memory (beyond about 4700 offsets) are walked
+// one node at a time: k_colour_walk with the colours in shared or global
+// memory, k_colour_walk_ext with the colours in an extended array read through
+// L1 and two nodes in flight per barrier.
 #include <limits.h>
 #include <string.h>
 
@@ -213,7 +213,8 @@ static int prep(pt_ctx *c, const int dims[4], int mu, const int *p_list, int n_p
     Geom g = make_geom(dims);
     cp.n_off = (int)(st.size() / 4);
     PT_CHECK_ARG(cp.n_off < 60000, "colouring: stencil of %d offsets exceeds the 16-bit colour range", cp.n_off);
-    size_t off_b = ((size_t)cp.n_off * sizeof(int4) + 255) & ~(size_t)255;
+    // the int4 stencil, or the walk's packed offsets and its first[t] table
+    size_t off_b = ((size_t)cp.n_off * sizeof(int4) + (size_t)dims[3] * sizeof(int) + 255) & ~(size_t)255;
     size_t vis_b = with_visit ? (((size_t)g.N * sizeof(int) + 255) & ~(size_t)255) : 0;
     void *ws;
     int rc = pt_workspace(c, off_b + vis_b + 256, &ws);
@@ -229,12 +230,13 @@ static int prep(pt_ctx *c, const int dims[4], int mu, const int *p_list, int n_p
             for (int i = 0; i < g.N; ++i) vis[i] = i;
         } else {
             size_t n = 0;
-            for (int pass = 0; pass < 2; ++pass)
-                for (int i = 0; i < g.N; ++i) {
-                    int r = i, s = 0;
-                    for (int nu = 0; nu < 4; ++nu) { s += r % dims[nu]; r /= dims[nu]; }
-                    if ((s & 1) == pass) vis[n++] = i;
-                }
+            for (int pass = 0; pass < 2; ++pass) {
+                int row = 0;
+                for (int t = 0; t < dims[3]; ++t)
+                    for (int z = 0; z < dims[2]; ++z)
+                        for (int y = 0; y < dims[1]; ++y, row += dims[0])
+                            for (int x = (pass ^ (y + z + t)) & 1; x < dims[0]; x += 2) vis[n++] = row + x;
+            }
         }
         PT_CUDA(cudaMemcpyAsync(cp.d_visit, vis.data(), vis.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
         // the host vector must outlive the copy
@@ -389,6 +391,294 @@ __global__ void __launch_bounds__(PT_EXT_NT, 1) k_colour_walk_ext(Geom g, ExtGeo
     }
 }
 
+// ------------------------------------------------------------ windowed walk
+// The same walk with 31 nodes in flight.  The visit order is cut into windows
+// of 31 nodes.  While warp 0 finds the colours of window n one node after the
+// other, each of the other 31 warps gathers the neighbourhood of one node of
+// window n + 1 from the colours committed so far (windows before n) into a
+// bitmap of the colours seen, and tests which nodes of windows n and n + 1 the
+// node is a neighbour of (the L1 distance to the nearer displaced image,
+// Eq. (8)).  At the end of a step the colours of window n enter the bitmaps of
+// the neighbours in window n + 1 and are committed.  The colour of a node is
+// then the first zero bit of its bitmap once the earlier nodes of its own
+// window have been entered: what the sequential definition gives.
+//
+// One node per step (k_colour_walk: 1024 threads on one neighbourhood) spent
+// its time on two barriers and a search per node, 1.0 to 1.3 us whatever the
+// stencil; here the gathers of 31 nodes overlap and only the search is serial.
+// Measured, one node per step -> windowed: 16^4, (p, k) = (2, 4), red-black
+// 87.8 -> 8.8 ms; 16^3 x 32, (4, 2), natural 168 -> 8.5 ms; (4, 1) on 16^4,
+// where no two nodes of a window are neighbours, 3.6 ms.  What bounds it: the
+// issue slots of one SM (about 250 instructions per node besides the
+// neighbourhood) and, where a window's nodes neighbour each other, the search.
+// Skipping later nodes' offsets (win_range) took (2, 4) from 12.4 to 10.2 ms,
+// and the lists of win_resolve instead of a scan of the row per node to 8.8.
+//
+// COLT: colour type in shared memory (8 bits while the stencil has at most 254
+// offsets, so that no colour reaches 255); EXT: the colours of a larger
+// lattice in an extended array in global memory, read through L1 (ExtGeom).
+#define PT_WIN 31
+struct WinPar {
+    int n_off, NS, NW;         // offsets; stamp bytes per warp; words per bitmap row (odd: rows spread over banks)
+    unsigned add, sub;         // packed 128 - D and D per byte
+    unsigned short st[4];      // strides
+    int g0, nE, redblack;      // offsets to visit (below); redblack: every side even, red-black order
+};
+
+// Neighbours later in the visit order have no colour, so a node skips most of
+// their offsets.  The offsets are sorted by their t part (reduced to [0, D_3)):
+// from a node at t, a part o3 > 0 that stays below D_3 - t leads to a later
+// t plane, and a larger one wraps to an earlier plane.  So the walk in storage
+// order visits the g0 offsets with o3 = 0 and those from first[t] on.  In
+// red-black order with every side even the same holds among the offsets that
+// keep the parity (sorted first, nE of them); the others lead to the other
+// parity, all of it uncoloured while the even sites are walked and coloured
+// when the odd ones are.  (Red-black with an odd side: first[t] = g0, all.)
+__device__ __forceinline__ int win_range(const WinPar &wp, const int *first, int t, int par, int *skip) {
+    const int lb = first[t];
+    *skip = lb - wp.g0;
+    return (wp.redblack && !par ? wp.nE : wp.n_off) - *skip;
+}
+
+// linear index of packed coordinates; x + o (bytes below 2 D <= 254: no
+// carries), minus D in the bytes that reached D
+__device__ __forceinline__ unsigned win_site(const WinPar &wp, unsigned sm) {
+    const unsigned hb = (sm + wp.add) & 0x80808080u;
+    sm -= wp.sub & ((hb - (hb >> 7)) | hb);
+    return (sm & 0xffu) + ((sm >> 8) & 0xffu) * wp.st[1] + ((sm >> 16) & 0xffu) * wp.st[2] + (sm >> 24) * wp.st[3];
+}
+
+// The colours of a window's nodes, node i at lane i (-1 beyond cnt): `own` has
+// a bit for every earlier node of the window that is a neighbour, row the
+// lane's bitmap in shared memory.  Lane i holds the first four zeros of its
+// row; a node's colour is its first, and the later nodes that neighbour it
+// strike that colour from their lists: one shuffle and four selects per node.
+// A node whose list has run out when its turn comes has the lists filled anew
+// from the rows, into which the colours found so far are entered first.
+__device__ __forceinline__ void win_fill(const unsigned *row, int nw, int z[4]) {
+    int n = 0;
+    z[0] = z[1] = z[2] = z[3] = -1;
+    for (int q = 0; q < nw && n < 4; ++q) {
+        unsigned f = ~row[q];
+        while (f && n < 4) {
+            const int c = 32 * q + __ffs(f) - 1;
+            f &= f - 1;
+            if (n == 0) z[0] = c;
+            else if (n == 1) z[1] = c;
+            else if (n == 2) z[2] = c;
+            else z[3] = c;
+            ++n;
+        }
+    }
+}
+
+__device__ __forceinline__ int win_resolve(unsigned *row, int nw, unsigned own, int cnt) {
+    const int lane = threadIdx.x & 31;
+    int z[4] = {-1, -1, -1, -1};
+    if (lane < cnt) win_fill(row, nw, z);
+    if (!__any_sync(0xffffffffu, own != 0)) return z[0];
+    int mine = -1, entered = 0;              // entered: nodes whose colours are in the rows
+    for (int i = 0; i < cnt; ++i) {
+        int c = __shfl_sync(0xffffffffu, z[0], i);
+        if (c < 0) {
+            for (; entered < i; ++entered) {
+                const int ce = __shfl_sync(0xffffffffu, mine, entered);
+                if ((own >> entered) & 1u) row[ce >> 5] |= 1u << (ce & 31);
+            }
+            if (lane >= i && lane < cnt) win_fill(row, nw, z);
+            c = __shfl_sync(0xffffffffu, z[0], i);
+        }
+        if (lane == i) mine = c;
+        const int ci = ((own >> i) & 1u) ? c : -2;
+        const bool p1 = ci == z[0], p2 = p1 || ci == z[1], p3 = p2 || ci == z[2], p4 = p3 || ci == z[3];
+        z[0] = p1 ? z[1] : z[0];
+        z[1] = p2 ? z[2] : z[1];
+        z[2] = p3 ? z[3] : z[2];
+        z[3] = p4 ? -1 : z[3];
+    }
+    return mine;
+}
+
+template <typename COLT, bool EXT, bool NESTED>
+__global__ void __launch_bounds__(1024, 1) k_colour_window(Geom g, ExtGeom eg, WinPar wp, const int *__restrict__ off_g,
+                                                           const int *__restrict__ first,
+                                                           const int *__restrict__ visit, unsigned short *colext,
+                                                           int32_t *col, int *out, const int32_t *__restrict__ parent) {
+    extern __shared__ unsigned smem_w[];
+    unsigned *bm = smem_w;                                              // [2][PT_WIN][NW]
+    int *soff = reinterpret_cast<int *>(bm + 2 * PT_WIN * wp.NW);       // [n_off]
+    unsigned char *stamps = reinterpret_cast<unsigned char *>(soff + ((wp.n_off + 3) & ~3));
+    unsigned *nbr = reinterpret_cast<unsigned *>(stamps + (size_t)PT_WIN * wp.NS);   // bit d: offset d is in the stencil
+    COLT *scol = reinterpret_cast<COLT *>(nbr + (g.N + 31) / 32);
+    __shared__ unsigned s_own[2][32];      // earlier neighbours of each node within its window
+    __shared__ int s_col[2][32], s_m[2], s_nw[2];
+    constexpr COLT NONE = (COLT)~(COLT)0;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    for (int o = tid; o < wp.n_off; o += 1024) soff[o] = off_g[o];
+    for (int i = tid; i < PT_WIN * wp.NS / 4; i += 1024) reinterpret_cast<unsigned *>(stamps)[i] = 0;
+    if (!EXT) {
+        for (int i = tid; i < g.N; i += 1024) scol[i] = NONE;
+        for (int i = tid; i < (g.N + 31) / 32; i += 1024) nbr[i] = 0;
+    }
+    if (tid < 2) { s_m[tid] = 0; s_nw[tid] = 0; }
+    __syncthreads();
+    if (!EXT)
+        for (int o = tid; o < wp.n_off; o += 1024) {
+            const unsigned d = win_site(wp, (unsigned)soff[o]);
+            atomicOr(&nbr[d >> 5], 1u << (d & 31));
+        }
+    __syncthreads();
+    const int n_win = (g.N + PT_WIN - 1) / PT_WIN;
+    const int w = warp - 1;                // this warp's node of the window (warps 1 to 31)
+    unsigned char *stamp = stamps + (size_t)max(w, 0) * wp.NS;
+    // nodes of windows n + 1 and n at this lane (-1: none) and their coordinates (packed unless EXT)
+    int v_next = (lane < PT_WIN && lane < g.N) ? visit[lane] : -1, v_cur = -1;
+    int xc[4] = {0, 0, 0, 0};
+    unsigned xpc = 0;
+    int m = 0;                             // warp 0: colours used so far
+    for (int n = -1; n < n_win; ++n) {
+        const int a = n & 1, b = (n + 1) & 1;
+        bool adj_prev = false;
+        int v_new = -1, xn[4] = {0, 0, 0, 0};
+        unsigned xpn = 0;
+        if (warp == 0) {
+            if (n >= 0) {
+                // ---- the colours of window n
+                const int cnt = min(PT_WIN, g.N - n * PT_WIN), nw = s_nw[a];
+                const unsigned own = lane < cnt ? s_own[a][lane] : 0u;
+                unsigned *rows = bm + a * PT_WIN * wp.NW;
+                const int mine = win_resolve(rows + min(lane, PT_WIN - 1) * wp.NW, nw, own, cnt);
+                m = max(m, __reduce_max_sync(0xffffffffu, mine + 1));
+                s_col[a][lane] = mine;
+                if (lane == 0) s_m[a] = m;
+            }
+        } else if (n + 1 < n_win) {
+            // ---- the neighbourhood of node w of window n + 1
+            const int t0 = (n + 1) * PT_WIN;
+            if (t0 + PT_WIN + lane < g.N && lane < PT_WIN) v_new = visit[t0 + PT_WIN + lane];
+            int xv[4];
+            site_coords(g, max(v_next, 0), xv);
+            const unsigned xpv = (unsigned)xv[0] | (unsigned)xv[1] << 8 | (unsigned)xv[2] << 16 | (unsigned)xv[3] << 24;
+            const int vw = __shfl_sync(0xffffffffu, v_next, w);
+            const int nw = min(wp.NW, ((s_m[a ^ 1] + 2 * PT_WIN) >> 5) + 1);    // s_m: as of window n - 1
+            if (vw >= 0) {                                              // (vw is the same in every lane)
+                const int step = n + 1;
+                const unsigned char tag = (unsigned char)(1 + step % 255);
+                if (step && step % 255 == 0)
+                    for (int i = lane; i < wp.NS / 4; i += 32) reinterpret_cast<unsigned *>(stamp)[i] = 0;
+                __syncwarp();
+                const int pw = NESTED ? parent[vw] : 0;
+                bool adj_own;
+                int xb = 0, t, par;
+                unsigned xp = 0;
+                if (EXT) {
+                    int xw[4];
+#pragma unroll
+                    for (int nu = 0; nu < 4; ++nu) xw[nu] = __shfl_sync(0xffffffffu, xv[nu], w);
+                    adj_prev = v_cur >= 0 && ext_neighbour(g, eg, xc, xw);
+                    adj_own = lane < w && v_next >= 0 && ext_neighbour(g, eg, xv, xw);
+                    xb = ext_base(eg, xw);
+                    t = xw[3];
+                    par = (xw[0] + xw[1] + xw[2] + xw[3]) & 1;
+                } else {
+                    // the difference of two nodes, reduced, is in the stencil or not
+                    xp = __shfl_sync(0xffffffffu, xpv, w);
+                    const unsigned dp = win_site(wp, xp + (wp.sub - xpc)), dn = win_site(wp, xp + (wp.sub - xpv));
+                    adj_prev = v_cur >= 0 && ((nbr[dp >> 5] >> (dp & 31)) & 1u);
+                    adj_own = lane < w && v_next >= 0 && ((nbr[dn >> 5] >> (dn & 31)) & 1u);
+                    t = (int)(xp >> 24);
+                    par = (int)(xp + (xp >> 8) + (xp >> 16) + (xp >> 24)) & 1;
+                }
+                int skip;
+                const int n_vis = win_range(wp, first, t, par, &skip);
+                if (NESTED) {
+                    adj_prev = adj_prev && parent[max(v_cur, 0)] == pw;
+                    adj_own = adj_own && parent[max(v_next, 0)] == pw;
+                }
+                const unsigned own = __ballot_sync(0xffffffffu, adj_own);
+                if (lane == 0) s_own[b][w] = own;
+                constexpr int UN = 4;
+                for (int o0 = lane; o0 < n_vis; o0 += 32 * UN) {
+                    COLT cv[UN];
+#pragma unroll
+                    for (int u = 0; u < UN; ++u) {
+                        const int o = o0 + 32 * u;
+                        cv[u] = NONE;
+                        if (o < n_vis) {
+                            const int off = soff[o < wp.g0 ? o : o + skip];
+                            if (EXT) {
+                                cv[u] = (COLT)colext[xb + off];
+                            } else {
+                                const unsigned y = win_site(wp, xp + (unsigned)off);
+                                cv[u] = scol[y];
+                                if (NESTED && parent[y] != pw) cv[u] = NONE;
+                            }
+                        }
+                    }
+#pragma unroll
+                    for (int u = 0; u < UN; ++u)
+                        if (cv[u] != NONE) stamp[cv[u]] = tag;
+                }
+                __syncwarp();
+                unsigned *row = bm + (b * PT_WIN + w) * wp.NW;
+                for (int q0 = 0; q0 < nw; q0 += 32) {
+                    unsigned word = 0;
+                    for (int q = q0; q < min(nw, q0 + 32); ++q) {
+                        const unsigned bb = __ballot_sync(0xffffffffu, 32 * q + lane < wp.NS && stamp[32 * q + lane] == tag);
+                        if (lane == q - q0) word = bb;
+                    }
+                    if (q0 + lane < nw) row[q0 + lane] = word;
+                }
+            }
+            if (tid == 32) s_nw[b] = nw;
+#pragma unroll
+            for (int nu = 0; nu < 4; ++nu) xn[nu] = xv[nu];
+            xpn = xpv;
+        }
+        __syncthreads();
+        if (warp > 0) {
+            // ---- window n enters the rows of window n + 1 and is committed
+            if (adj_prev) {
+                const int c = s_col[a][lane];
+                atomicOr(&bm[(b * PT_WIN + w) * wp.NW + (c >> 5)], 1u << (c & 31));
+            }
+            const int i = __shfl_sync(0xffffffffu, v_cur, w);
+            if (i >= 0) {
+                const int f = s_col[a][w];
+                if (EXT) {
+                    int x[4];
+#pragma unroll
+                    for (int nu = 0; nu < 4; ++nu) x[nu] = __shfl_sync(0xffffffffu, xc[nu], w);
+                    if (lane < 16) {
+                        int e = 0, ok = 1;
+#pragma unroll
+                        for (int nu = 0; nu < 4; ++nu) {
+                            int ev = x[nu] - eg.lo[nu];                 // in [0, 2D): one reduction
+                            ev -= (ev >= g.D[nu]) ? g.D[nu] : 0;
+                            ev += ((lane >> nu) & 1) * g.D[nu];
+                            ok &= ev < eg.E[nu];
+                            e += ev * eg.ES[nu];
+                        }
+                        if (ok) colext[e] = (unsigned short)f;
+                    }
+                    if (lane == 0) col[i] = f;
+                } else if (lane == 0) {
+                    scol[i] = (COLT)f;
+                }
+            }
+            v_cur = v_next;
+            v_next = v_new;
+#pragma unroll
+            for (int nu = 0; nu < 4; ++nu) xc[nu] = xn[nu];
+            xpc = xpn;
+        }
+        __syncthreads();
+    }
+    if (!EXT)
+        for (int i = tid; i < g.N; i += 1024) col[i] = (int32_t)scol[i];
+    if (tid == 0) out[0] = m;
+}
+
 // Offsets of the walk: reduced modulo the lattice, merged, x itself dropped,
 // packed (see walk_site).  Sides are below 65536 (PT_CHECK in the caller).
 static std::vector<uint2> walk_offsets(const std::vector<int> &st, const int dims[4]) {
@@ -430,7 +720,6 @@ static int colour_walk(pt_ctx *c, const int dims[4], int mu, const int *p_list, 
     const int n_off = (int)wo.size();
     // the packed offsets take the place of the int4 stencil in the workspace (8 <= 16 bytes per row)
     uint2 *d_off = reinterpret_cast<uint2 *>(cp.d_off);
-    if (n_off) PT_CUDA(cudaMemcpyAsync(d_off, wo.data(), wo.size() * sizeof(uint2), cudaMemcpyHostToDevice, c->stream));
     // a node's colour never exceeds its number of neighbours: stamps for 0..n_off
     const int n_stamp = n_off + 2;
     const size_t stamp_b = (size_t)((n_stamp + 1) & ~1) * sizeof(int);
@@ -443,14 +732,78 @@ static int colour_walk(pt_ctx *c, const int dims[4], int mu, const int *p_list, 
     const bool sh_col = stamp_b + col_b <= (size_t)max_smem;
     const bool sh_off = stamp_b + off_b + (sh_col ? col_b : 0) <= (size_t)max_smem;
     size_t shared_b = stamp_b + (sh_off ? off_b : 0) + (sh_col ? col_b : 0);
-    // large lattices: the extended-array walk (two stamp buffers in shared memory, deltas in registers)
+    ExtGeom eg;
+    eg.mu = mu;
+    eg.k = k;
+    eg.n_p = n_p;
+    for (int n = 0; n < n_p; ++n) eg.p[n] = p_list[n] % dims[mu];
+    // the windowed walk wherever its stamps and rows (about 45 bytes per offset) fit: colours in shared
+    // memory while they fit beside them, else in the extended array (not nested: its parents are by site)
+    WinPar wp;
+    memset(&wp, 0, sizeof(wp));
+    wp.n_off = n_off;
+    wp.NS = (n_off + 2 + 31) / 32 * 32;
+    wp.NW = (wp.NS / 32 + 1) | 1;
+    const size_t win_b = (size_t)2 * PT_WIN * wp.NW * sizeof(unsigned) + (size_t)((n_off + 3) & ~3) * sizeof(int) +
+                         (size_t)PT_WIN * wp.NS;
+    bool bytes_ok = (long)dims[0] * dims[1] * dims[2] <= 65535;
+    for (int nu = 0; nu < 4; ++nu) {
+        bytes_ok = bytes_ok && dims[nu] <= 127;
+        wp.add |= (unsigned)(128 - std::min(dims[nu], 127)) << (8 * nu);
+        wp.sub |= (unsigned)std::min(dims[nu], 127) << (8 * nu);
+        wp.st[nu] = (unsigned short)g.stride[nu];
+    }
+    const size_t nbr_b = (size_t)((g.N + 31) / 32) * sizeof(unsigned);
+    const bool win8 = bytes_ok && n_off <= 254 && win_b + nbr_b + (size_t)g.N <= (size_t)max_smem;
+    const bool win16 = bytes_ok && win_b + nbr_b + (size_t)g.N * 2 <= (size_t)max_smem;
+    const bool win_ext = !parent && win_b <= (size_t)max_smem;
+    // offsets in the order the windowed walk visits them (win_range), and its table
+    std::vector<int> first(dims[3]);
+    int *d_first = reinterpret_cast<int *>((char *)cp.d_off + (size_t)cp.n_off * sizeof(int4));
+    if (win8 || win16 || win_ext) {
+        const bool even = dims[0] % 2 == 0 && dims[1] % 2 == 0 && dims[2] % 2 == 0 && dims[3] % 2 == 0;
+        wp.redblack = order == PT_ORDER_REDBLACK && even;
+        auto odd = [](const uint2 &o) { return ((o.x ^ (o.x >> 16) ^ o.y ^ (o.y >> 16)) & 1u) != 0; };
+        if (wp.redblack) std::stable_partition(wo.begin(), wo.end(), [&](const uint2 &o) { return !odd(o); });
+        wp.nE = n_off;
+        if (wp.redblack) wp.nE = (int)std::count_if(wo.begin(), wo.end(), [&](const uint2 &o) { return !odd(o); });
+        wp.g0 = 0;
+        while (wp.g0 < wp.nE && (wo[wp.g0].y >> 16) == 0) ++wp.g0;
+        int lb = wp.nE;
+        for (int t = 0; t < dims[3]; ++t) {
+            while (lb > wp.g0 && (int)(wo[lb - 1].y >> 16) >= dims[3] - t) --lb;
+            first[t] = order == PT_ORDER_REDBLACK && !even ? wp.g0 : lb;
+        }
+        PT_CUDA(cudaMemcpyAsync(d_first, first.data(), first.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
+    }
+    if (win8 || win16) {
+        std::vector<int> po(n_off);
+        for (int i = 0; i < n_off; ++i)
+            po[i] = (int)((wo[i].x & 0xffu) | (wo[i].x >> 16) << 8 | (wo[i].y & 0xffu) << 16 | (wo[i].y >> 16) << 24);
+        int *d_po = reinterpret_cast<int *>(cp.d_off);
+        if (n_off) PT_CUDA(cudaMemcpyAsync(d_po, po.data(), po.size() * sizeof(int), cudaMemcpyHostToDevice, c->stream));
+        const size_t smem = win_b + nbr_b + (size_t)g.N * (win8 ? 1 : 2);
+#define PT_WINDOW(T, NE)                                                                                         \
+    do {                                                                                                         \
+        PT_CUDA(cudaFuncSetAttribute(k_colour_window<T, false, NE>, cudaFuncAttributeMaxDynamicSharedMemorySize,  \
+                                     (int)smem));                                                                \
+        k_colour_window<T, false, NE><<<1, 1024, smem, c->stream>>>(g, eg, wp, d_po, d_first, cp.d_visit, nullptr, \
+                                                                    col_dev, cp.d_out, parent);                  \
+    } while (0)
+        if (win8) { if (parent) PT_WINDOW(unsigned char, true); else PT_WINDOW(unsigned char, false); }
+        else { if (parent) PT_WINDOW(unsigned short, true); else PT_WINDOW(unsigned short, false); }
+#undef PT_WINDOW
+        ++pt_kernel_launch_count;
+        PT_CUDA(cudaGetLastError());
+        PT_CUDA(cudaMemcpyAsync(c->h_flags, cp.d_out, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+        PT_CUDA(cudaStreamSynchronize(c->stream));
+        *n_colours = c->h_flags[0];
+        return PT_OK;
+    }
+    // larger lattices or stencils: the extended array, walked in windows or (stencils whose stamps do not
+    // fit 31 times) one node per barrier with two stamp buffers and the deltas in registers
     const size_t ext_smem = (size_t)(2 * n_stamp) * sizeof(int);
-    if (!parent && !sh_col && ext_smem <= (size_t)max_smem && n_p <= 64 && n_off <= PT_EXT_NT * 24) {
-        ExtGeom eg;
-        eg.mu = mu;
-        eg.k = k;
-        eg.n_p = n_p;
-        for (int n = 0; n < n_p; ++n) eg.p[n] = p_list[n] % dims[mu];
+    if (win_ext || (!parent && !sh_col && ext_smem <= (size_t)max_smem && n_p <= 64 && n_off <= PT_EXT_NT * 24)) {
         // per dimension: signed offsets if the largest minimal image R fits (2R + 1 <= D), else [0, D)
         int sgn[4];
         long E = 1;
@@ -495,7 +848,13 @@ static int colour_walk(pt_ctx *c, const int dims[4], int mu, const int *p_list, 
         k_colour_walk_ext<U><<<1, PT_EXT_NT, ext_smem, c->stream>>>(g, eg, d_delta, n_off, cp.d_visit, d_ext,    \
                                                                     col_dev, n_stamp, cp.d_out);                 \
     } while (0)
-        if (n_off <= PT_EXT_NT * 4) PT_EXT(4);
+        if (win_ext) {
+            PT_CUDA(cudaFuncSetAttribute(k_colour_window<unsigned short, true, false>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)win_b));
+            k_colour_window<unsigned short, true, false><<<1, 1024, win_b, c->stream>>>(
+                g, eg, wp, d_delta, d_first, cp.d_visit, d_ext, col_dev, cp.d_out, nullptr);
+        }
+        else if (n_off <= PT_EXT_NT * 4) PT_EXT(4);
         else if (n_off <= PT_EXT_NT * 8) PT_EXT(8);
         else if (n_off <= PT_EXT_NT * 12) PT_EXT(12);
         else if (n_off <= PT_EXT_NT * 16) PT_EXT(16);
@@ -511,6 +870,7 @@ static int colour_walk(pt_ctx *c, const int dims[4], int mu, const int *p_list, 
         *n_colours = c->h_flags[0];
         return PT_OK;
     }
+    if (n_off) PT_CUDA(cudaMemcpyAsync(d_off, wo.data(), wo.size() * sizeof(uint2), cudaMemcpyHostToDevice, c->stream));
 #define PT_WALK(SC, SO, NE)                                                                                      \
     do {                                                                                                         \
         PT_CUDA(cudaFuncSetAttribute(k_colour_walk<SC, SO, NE>, cudaFuncAttributeMaxDynamicSharedMemorySize,      \
