@@ -27,6 +27,7 @@
 #include <vector>
 
 #include "engine.cuh"
+#include "fixed.cuh"
 
 #define PT_BLOCK 256        // threads per engine work item
 
@@ -44,6 +45,7 @@ struct Slot {
 struct EP {
     Geom g;
     int kind, nsb, R, gs, vec4;
+    int prec;                  // storage precision of the inner vectors (PT_PREC_*)
     int bs, spt;               // threads of an item kernel's CTA; sites per thread (an item is bs x spt sites)
     int eo;                    // Laplacian on the even Schur complement (inner vectors on the even sites)
     int nsite;                 // entries of a slot field: N, or N / 2 in even-odd mode
@@ -63,6 +65,9 @@ struct EP {
     int clover;                // even-odd Wilson with a clover term: the packed chiral blocks below
     const float4 *CL32;        // 1 + C (even), (1 + C)^{-1} (odd) for FP32 / BF16 inner storage
     const double2 *CL64;       // the same in FP64 (and 1 + C on the odd sites)
+    const int4 *Ufx;           // even-odd Wilson: links as fixed-point digits (fixed.cuh), even-odd order
+    const int *fx_em;          // and their exponent
+    int *fx_ex, *fx_et;        // exponents of the fixed-point x64 (even entries) and t64 (odd) [R][nsite]
     int mode;
     const int32_t *col;
     uint64_t seed;
@@ -73,7 +78,7 @@ struct EP {
     const double *B_user;      // solve mode: user layout sources
     double *X_user;            // solve mode: user layout solutions
     double *x64;
-    double *t64;               // even-odd: H_oe x64 (Laplacian) / D_oe x64 (Wilson) on the odd sites (FP64)
+    double *t64;               // even-odd: H_oe x64 (Laplacian, FP64) / D_oe x64 (Wilson, fixed point) on the odd sites
     double *b64;               // even-odd: b'_e of the slot's task (FP64; b_e + H_eo b_o / d, resp. + kappa D_eo b_o)
     void *e, *r, *pv, *q, *s, *t, *r0, *p1;   // p1: second CG direction buffer; even-odd: t = H_oe p (odd sites)
     Slot *slots;
@@ -1644,8 +1649,8 @@ __device__ __forceinline__ void wilson_hop_dir(const Geom &g, const LS *U, int a
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
                 Cx<R> t = cmul(u[a][0], h[k][0]);
-                t = cadd(t, cmul(u[a][1], h[k][1]));
-                t = cadd(t, cmul(u[a][2], h[k][2]));
+                t = cmac(t, u[a][1], h[k][1]);
+                t = cmac(t, u[a][2], h[k][2]);
                 uh[k][a] = t;
             }
         spin_accumulate<R>(mu, R(-1), eta, uh, acc);
@@ -1658,8 +1663,8 @@ __device__ __forceinline__ void wilson_hop_dir(const Geom &g, const LS *U, int a
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
                 Cx<R> t = cconjmul(u[0][a], h[k][0]);
-                t = cadd(t, cconjmul(u[1][a], h[k][1]));
-                t = cadd(t, cconjmul(u[2][a], h[k][2]));
+                t = cconjmac(t, u[1][a], h[k][1]);
+                t = cconjmac(t, u[2][a], h[k][2]);
                 uh[k][a] = t;
             }
         spin_accumulate<R>(mu, R(1), eta, uh, acc);
@@ -1703,8 +1708,8 @@ __device__ __forceinline__ void wilson_hop_fetch(const Geom &g, Fetch fetch, con
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
                     Cx<R> t = cmul(u[a][0], h[k][0]);
-                    t = cadd(t, cmul(u[a][1], h[k][1]));
-                    t = cadd(t, cmul(u[a][2], h[k][2]));
+                    t = cmac(t, u[a][1], h[k][1]);
+                    t = cmac(t, u[a][2], h[k][2]);
                     uh[k][a] = t;
                 }
             spin_accumulate<R>(mu, R(-1), eta, uh, acc);
@@ -1721,8 +1726,8 @@ __device__ __forceinline__ void wilson_hop_fetch(const Geom &g, Fetch fetch, con
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
                     Cx<R> t = cconjmul(u[0][a], h[k][0]);
-                    t = cadd(t, cconjmul(u[1][a], h[k][1]));
-                    t = cadd(t, cconjmul(u[2][a], h[k][2]));
+                    t = cconjmac(t, u[1][a], h[k][1]);
+                    t = cconjmac(t, u[2][a], h[k][2]);
                     uh[k][a] = t;
                 }
             spin_accumulate<R>(mu, R(1), eta, uh, acc);
@@ -1884,42 +1889,216 @@ __global__ void __launch_bounds__(PT_BLOCK, weo_minb<S>(2 * CLV)) k_weo_apply2(E
     ITEM_LOOP_END
 }
 
-// outer step, part 1: t64 = D_oe x64 at the odd entries (FP64); a new task
-// starts from x = 0, so its t64 is zero (written, not hopped: the
-// contraction reads it if the task converges at once)
-__global__ void __launch_bounds__(PT_BLOCK) k_weo_outer_hop(EP P) {
+// The outer step forms r = b'_e - S x64 with its two hops in block fixed point
+// (fixed.cuh): FP64 multiply-adds bound it before (about 1000 per entry and
+// hop at two per SM and cycle; ncu: FP64 pipe 86 % busy), and only the update,
+// the last subtraction and the sums are left on that pipe.  16^3 x 32, 48
+// right-hand sides, per outer step: hop 5.09 -> 1.76 ms, residual 6.04 -> 2.01 ms
+// (at 128 registers, 2 CTAs per SM, 0.5 KB of spills; without spills at one
+// CTA per SM 1.92 and 2.60 ms).  What bounds them: the integer pipes, each 64
+// lanes per SM and cycle (3400 multiply-adds and moves, 2900 additions, shifts
+// and selects per entry).
+//
+// The fixed-point copy of x64 lives in the inner vectors that an outer step
+// does not need (the next cycle starts from r alone): v, and as many of s, t
+// and the hop buffer as their storage type makes necessary.
+// Each vector takes 12, 6 or 3 of the components (8-, 4- or 2-byte storage).
+__device__ __forceinline__ FxField fx_x64(const EP &P, int j) {
+    const int b = P.prec == PT_PREC_FP64 ? 8 : P.prec == PT_PREC_MIXED_FP32 ? 4 : 2;
+    void *const v[4] = {P.q, P.s, P.t, P.p1};
+    FxField f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        char *base = (char *)(b == 8 ? v[0] : b == 4 ? v[i / 2] : v[i]) + (size_t)j * P.L * b;
+        f.p[i] = reinterpret_cast<longlong2 *>(base) + (size_t)(b == 8 ? 3 * i : b == 4 ? 3 * (i % 2) : 0) * P.nsite;
+    }
+    f.e = P.fx_ex + (size_t)j * P.nsite;
+    return f;
+}
+__device__ __forceinline__ FxField fx_t64(const EP &P, int j) {
+    const longlong2 *t = reinterpret_cast<const longlong2 *>(P.t64 + (size_t)j * P.L);
+    FxField f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) f.p[i] = t + (size_t)3 * i * P.nsite;
+    f.e = P.fx_et + (size_t)j * P.nsite;
+    return f;
+}
+
+__device__ __forceinline__ void fx_load(const longlong2 *q, int N, int h, FxC (&ps)[4][3]) {
+#pragma unroll
+    for (int c = 0; c < 12; ++c) {
+        const longlong2 v = q[(size_t)c * N + h];
+        ps[c / 3][c % 3] = FxC{v.x, v.y};
+    }
+}
+
+// x64 += e (x64 = 0 for a new task) and its fixed-point form
+template <typename S>
+__global__ void __launch_bounds__(PT_BLOCK) k_weo_outer_update(EP P) {
+    typedef typename ArithT<S>::T R;
     const int N = P.nsite;
     ITEM_LOOP(LIST_OUTER)
         const int ph = P.slots[j].phase;
         if (ph != PH_START && ph != PH_OUTER) continue;
-        const double *x = P.x64 + (size_t)j * P.L;
-        double *t = P.t64 + (size_t)j * P.L;
+        double *x = P.x64 + (size_t)j * P.L;
+        const S *e = slot_cptr<S>(P.e, j, P.L);
+        const FxField fx = fx_x64(P, j);
         SITE_LOOP(1)
-            Cx<double> o[12];
+            Cx<double> v[12];
             if (ph == PH_START) {
 #pragma unroll
-                for (int c = 0; c < 12; ++c) o[c] = Cx<double>{0.0, 0.0};
-            } else {
-                int xc[4];
-                const int s = half_site(P.g, 1, idx, xc);
-                Cx<double> acc[4][3];
-                wilson_hop_fetch<double, double>(
-                    P.g, [&](int y, int, int, Cx<double> f[4][3]) { load_spinor<double, double>(x, N, y >> 1, f); },
-                    P.U64, P.antip, s, xc, acc);
-#pragma unroll
-                for (int c = 0; c < 12; ++c) o[c] = acc[c / 3][c % 3];
-                if (P.clover) clover_mul(P.CL64, N, 1, idx, o);      // t64 = A_oo^{-1} D_oe x64
+                for (int c = 0; c < 12; ++c) v[c] = Cx<double>{0.0, 0.0};
+                store_spinor<double, double>(x, N, idx, v);
+                continue;
             }
-            store_spinor<double, double>(t, N, idx, o);
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                Cx<R> ev[2];
+                ld_pair<S, R>(e, N, k, idx, ev);
+#pragma unroll
+                for (int w = 0; w < 2; ++w) {
+                    const Cx<double> xv = ld_cx<double, double>(x, N, 2 * k + w, idx);
+                    v[2 * k + w] = Cx<double>{xv.re + (double)ev[w].re, xv.im + (double)ev[w].im};
+                }
+            }
+            store_spinor<double, double>(x, N, idx, v);
+            FxC q[12];
+            P.fx_ex[(size_t)j * N + idx] = fx_site(v, q);
+#pragma unroll
+            for (int c = 0; c < 12; ++c)
+                const_cast<longlong2 *>(fx.p[c / 3])[(size_t)(c % 3) * N + idx] = make_longlong2(q[c].re, q[c].im);
         SITE_LOOP_END
     ITEM_LOOP_END
 }
 
-// outer step, part 2 (new tasks only), at the even entries: b'_e = b_e +
-// kappa D_eo b_o from the source regenerated at the site and at those of its
+// outer step, part 1: t64 = D_oe x64 at the odd entries (clover: A_oo^{-1}
+// D_oe x64); a new task starts from x = 0, so its t64 is zero (written, not
+// hopped: the contraction reads it if the task converges at once)
+__global__ void __launch_bounds__(PT_BLOCK, 2) k_weo_outer_hop(EP P) {
+    const int N = P.nsite;
+    const int ku = fx_link_exp(P.fx_em);
+    ITEM_LOOP(LIST_OUTER)
+        const int ph = P.slots[j].phase;
+        if (ph != PH_START && ph != PH_OUTER) continue;
+        const FxField fx = fx_x64(P, j);
+        longlong2 *t = reinterpret_cast<longlong2 *>(P.t64 + (size_t)j * P.L);
+        SITE_LOOP(1)
+            FxC acc[4][3];
+            int E = FX_ZERO;
+            if (ph == PH_START) {
+#pragma unroll
+                for (int c = 0; c < 12; ++c) acc[c / 3][c % 3] = FxC{0, 0};
+            } else {
+                int xc[4];
+                const int s = half_site(P.g, 1, idx, xc);
+                E = fx_hop(P.g, fx, P.Ufx, ku, P.antip, 1, s, xc, acc);
+                if (P.clover) {
+                    const double sc = fx_pow2(E);
+                    Cx<double> v[12];
+#pragma unroll
+                    for (int c = 0; c < 12; ++c)
+                        v[c] = Cx<double>{sc * (double)acc[c / 3][c % 3].re, sc * (double)acc[c / 3][c % 3].im};
+                    clover_mul(P.CL64, N, 1, idx, v);
+                    FxC q[12];
+                    E = fx_site(v, q);
+#pragma unroll
+                    for (int c = 0; c < 12; ++c) acc[c / 3][c % 3] = q[c];
+                } else {
+                    E = fx_normalise(acc, E);
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < 12; ++c)
+                t[(size_t)c * N + idx] = make_longlong2(acc[c / 3][c % 3].re, acc[c / 3][c % 3].im);
+            P.fx_et[(size_t)j * N + idx] = E;
+        SITE_LOOP_END
+    ITEM_LOOP_END
+}
+
+// u, rotated by a noise value z (+-1 or +-i) and negated if neg: exact
+__device__ __forceinline__ Cx<double> times_unit(Cx<double> u, Cx<double> z, bool neg) {
+    const bool im = z.im != 0.0;
+    const bool n = neg != ((im ? z.im : z.re) < 0.0);
+    const double a = im ? -u.im : u.re, b = im ? u.re : u.im;
+    return Cx<double>{neg_if(a, n), neg_if(b, n)};
+}
+
+// D_eo b_o at the even site s for a diluted probe: the source has one nonzero
+// component (spin sp, colour cl, a unit) at the sites of its colour class, so a
+// neighbour in the class adds one column of its link to spin sp and, through
+// the projector's off-diagonal entry, to one other spin.  No multiplication.
+__device__ __forceinline__ void weo_probe_hop(const EP &P, const Task &tk, uint64_t key, int s, const int xc[4],
+                                              Cx<double> (&own)[3], Cx<double> (&pa)[3], Cx<double> (&pb)[3]) {
+    const int sp = tk.comp / 3, cl = tk.comp % 3, N = P.g.N;
+    const int32_t *col = P.col + (size_t)tk.cidx * N;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) own[a] = pa[a] = pb[a] = Cx<double>{0.0, 0.0};
+#pragma unroll
+    for (int mu = 0; mu < 4; ++mu)
+#pragma unroll
+        for (int dir = 1; dir >= -1; dir -= 2) {
+            const int y = dir > 0 ? nb_fwd(P.g, s, xc, mu) : nb_bwd(P.g, s, xc, mu);
+            if (col[y] != tk.colour) continue;
+            const Cx<double> z = pt_noise(key, (uint64_t)y, P.noise);
+            const bool edge = P.antip && mu == 3 && xc[3] == (dir > 0 ? P.g.D[3] - 1 : 0);
+            // (1 - g_mu) forward, (1 + g_mu) backward: off-diagonal entry +-1 or +-i
+            const bool minus = mu == 0 ? sp >= 2 : mu == 1 ? (sp == 0 || sp == 3) : mu == 2 ? (sp == 1 || sp == 2) : false;
+            const bool neg = minus != (dir > 0);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                Cx<double> u;
+                if (dir > 0) {
+                    u = ld_cx<double, double>(P.U64, N, mu * 9 + 3 * a + cl, s);
+                } else {
+                    u = ld_cx<double, double>(P.U64, N, mu * 9 + 3 * cl + a, y);
+                    u.im = -u.im;
+                }
+                const Cx<double> w = times_unit(u, z, edge);
+                own[a] = cadd(own[a], w);
+                const Cx<double> v = (mu & 1) ? w : ctimes_i(w);
+                const Cx<double> vn = Cx<double>{neg_if(v.re, neg), neg_if(v.im, neg)};
+                if (mu < 2) pa[a] = cadd(pa[a], vn);         // spin 3 - sp
+                else pb[a] = cadd(pb[a], vn);                // spin sp ^ 2
+            }
+        }
+}
+
+// new tasks, at the even entries: b'_e = b_e + kappa D_eo b_o (clover: D_eo
+// A_oo^{-1} b_o) from the source regenerated at the site and at those of its
 // eight odd neighbours where it can be nonzero (a skipped neighbour would add
-// exact zeros); kept in FP64 for the task's later outer steps
+// exact zeros), kept in FP64 for the task's later outer steps; x = 0, so
+// r64 = b'_e, and r = (S) r64 starts the inner solve (p = r0 = r, e = 0).
+// Partials: |r64|^2, |b|^2 of both sites of the entry (even and odd), |r|^2 of
+// the rounded r (summed per entry in the inner solve's arithmetic).
+template <typename S>
+__device__ __forceinline__ void weo_start_entry(const EP &P, int j, int idx, const Cx<double> (&rv)[12], double v[3]) {
+    typedef typename ArithT<S>::T R;
+    const int N = P.nsite;
+    Cx<R> rs[12], zero[12];
+    R v2 = R(0);
+#pragma unroll
+    for (int c = 0; c < 12; ++c) {
+        v[0] += rv[c].re * rv[c].re + rv[c].im * rv[c].im;
+        rs[c] = Cx<R>{rnd<S, R>((R)rv[c].re), rnd<S, R>((R)rv[c].im)};
+        v2 += rs[c].re * rs[c].re + rs[c].im * rs[c].im;
+        zero[c] = Cx<R>{R(0), R(0)};
+    }
+    v[2] += (double)v2;
+    store_spinor<S, R>(slot_ptr<S>(P.r, j, P.L), N, idx, rs);
+    store_spinor<S, R>(slot_ptr<S>(P.pv, j, P.L), N, idx, rs);
+    store_spinor<S, R>(slot_ptr<S>(P.r0, j, P.L), N, idx, rs);
+    store_spinor<S, R>(slot_ptr<S>(P.e, j, P.L), N, idx, zero);
+}
+
+// (one build of the outer kernels serves every storage precision)
+__device__ __forceinline__ void weo_start_any(const EP &P, int j, int idx, const Cx<double> (&rv)[12], double v[3]) {
+    if (P.prec == PT_PREC_MIXED_FP32) weo_start_entry<float>(P, j, idx, rv, v);
+    else if (P.prec == PT_PREC_FP64) weo_start_entry<double>(P, j, idx, rv, v);
+    else weo_start_entry<__nv_bfloat16>(P, j, idx, rv, v);
+}
+
 __global__ void __launch_bounds__(PT_BLOCK) k_weo_outer_bprime(EP P) {
+    __shared__ double sh[32 * 3];
     const int N = P.nsite;
     const double kap = P.kappa;
     ITEM_LOOP(LIST_OUTER)
@@ -1928,121 +2107,108 @@ __global__ void __launch_bounds__(PT_BLOCK) k_weo_outer_bprime(EP P) {
         const Task tk = P.tasks[st.task];
         const uint64_t key = (P.mode == MODE_SOLVE) ? 0 : pt_set_key(P.seed, tk.set);
         double *bp = P.b64 + (size_t)j * P.L;
-        SITE_LOOP(1)
-            int xc[4];
-            const int s = half_site(P.g, 0, idx, xc);
-            Cx<double> acc[4][3], bv[12];
-#pragma unroll
-            for (int sp = 0; sp < 4; ++sp)
-#pragma unroll
-                for (int a = 0; a < 3; ++a) acc[sp][a] = Cx<double>{0.0, 0.0};
-#pragma unroll
-            for (int mu = 0; mu < 4; ++mu)
-#pragma unroll
-                for (int dir = 1; dir >= -1; dir -= 2) {
-                    const int y = dir > 0 ? nb_fwd(P.g, s, xc, mu) : nb_bwd(P.g, s, xc, mu);
-                    if (!source_may_be_nonzero(P, tk, y)) continue;
-                    int y4[4];
-                    nb_coords(P.g, xc, mu, dir, y4);
-                    Cx<double> f[4][3];
-                    if (P.clover) {                           // A_oo^{-1} b_o at the neighbour
-                        Cx<double> v[12];
-#pragma unroll
-                        for (int c = 0; c < 12; ++c) v[c] = source_val<1>(P, tk, key, y, y4, c);
-                        clover_mul(P.CL64, N, 1, y >> 1, v);
-#pragma unroll
-                        for (int c = 0; c < 12; ++c) f[c / 3][c % 3] = v[c];
-                    } else {
-#pragma unroll
-                        for (int c = 0; c < 12; ++c) f[c / 3][c % 3] = source_val<1>(P, tk, key, y, y4, c);
-                    }
-                    wilson_hop_dir<double, double>(P.g, P.U64, P.antip, s, xc, mu, dir > 0, f, acc);
-                }
-#pragma unroll
-            for (int c = 0; c < 12; ++c)
-                bv[c] = cadd(source_val<1>(P, tk, key, s, xc, c), cscale(acc[c / 3][c % 3], kap));
-            store_spinor<double, double>(bp, N, idx, bv);
-        SITE_LOOP_END
-    ITEM_LOOP_END
-}
-
-// outer step, part 3, at the even entries: r64 = b'_e - S x64 in FP64
-// (= b'_e for a new task, x = 0); r = (S) r64 starts the inner solve
-// (p = r0 = r, e = 0).  Partials: |r64|^2, |b|^2 of both sites of the entry
-// (even and odd; used when the task starts), |r|^2 of the rounded r.
-template <typename S>
-__global__ void __launch_bounds__(PT_BLOCK) k_weo_outer_residual(EP P) {
-    typedef typename ArithT<S>::T R;
-    __shared__ double sh[32 * 3];
-    const int N = P.nsite;
-    const double k2 = P.kappa * P.kappa;
-    ITEM_LOOP(LIST_OUTER)
-        const Slot &st = P.slots[j];
-        const int ph = st.phase;
-        if (ph != PH_START && ph != PH_OUTER) continue;
-        const Task tk = P.tasks[st.task];
-        const uint64_t key = (P.mode == MODE_SOLVE) ? 0 : pt_set_key(P.seed, tk.set);
-        S *r = slot_ptr<S>(P.r, j, P.L);
-        S *pv = slot_ptr<S>(P.pv, j, P.L);
-        S *r0 = slot_ptr<S>(P.r0, j, P.L);
-        S *e = slot_ptr<S>(P.e, j, P.L);
-        const double *x = P.x64 + (size_t)j * P.L;
-        const double *t = P.t64 + (size_t)j * P.L;
-        const double *bp = P.b64 + (size_t)j * P.L;
+        const bool plain_probe = P.mode == MODE_TRACE || !(P.mode == MODE_SOLVE || (tk.flags & TASK_ADJ));
+        const bool sparse = plain_probe && P.dilute && !P.clover;
         double v[3] = {0.0, 0.0, 0.0};
         SITE_LOOP(1)
             int xc[4];
             const int s = half_site(P.g, 0, idx, xc);
-            Cx<double> rv[12];
-            if (ph == PH_START) {
-                int xp[4] = {xc[0] ^ 1, xc[1], xc[2], xc[3]};          // the odd site of the same entry
-                Cx<double> bs[4][3];
-                load_spinor<double, double>(bp, N, idx, bs);
+            Cx<double> bv[12];
+            if (sparse) {
+                const int sp = tk.comp / 3, cl = tk.comp % 3;
+                Cx<double> own[3], pa[3], pb[3];
+                weo_probe_hop(P, tk, key, s, xc, own, pa, pb);
+                const bool in = P.col[(size_t)tk.cidx * P.g.N + s] == tk.colour;
+                const Cx<double> z = in ? pt_noise(key, (uint64_t)s, P.noise) : Cx<double>{0.0, 0.0};
+#pragma unroll
+                for (int c = 0; c < 12; ++c) {
+                    const int k = c / 3, a = c % 3;
+                    Cx<double> w = k == sp ? own[a] : k == 3 - sp ? pa[a] : k == (sp ^ 2) ? pb[a] : Cx<double>{0.0, 0.0};
+                    w = cscale(w, kap);
+                    bv[c] = (k == sp && a == cl) ? cadd(z, w) : w;
+                }
+            } else {
+                Cx<double> acc[4][3];
+#pragma unroll
+                for (int sp = 0; sp < 4; ++sp)
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) acc[sp][a] = Cx<double>{0.0, 0.0};
+#pragma unroll
+                for (int mu = 0; mu < 4; ++mu)
+#pragma unroll
+                    for (int dir = 1; dir >= -1; dir -= 2) {
+                        const int y = dir > 0 ? nb_fwd(P.g, s, xc, mu) : nb_bwd(P.g, s, xc, mu);
+                        if (!source_may_be_nonzero(P, tk, y)) continue;
+                        int y4[4];
+                        nb_coords(P.g, xc, mu, dir, y4);
+                        Cx<double> f[4][3];
+                        if (P.clover) {                           // A_oo^{-1} b_o at the neighbour
+                            Cx<double> w[12];
+#pragma unroll
+                            for (int c = 0; c < 12; ++c) w[c] = source_val<1>(P, tk, key, y, y4, c);
+                            clover_mul(P.CL64, N, 1, y >> 1, w);
+#pragma unroll
+                            for (int c = 0; c < 12; ++c) f[c / 3][c % 3] = w[c];
+                        } else {
+#pragma unroll
+                            for (int c = 0; c < 12; ++c) f[c / 3][c % 3] = source_val<1>(P, tk, key, y, y4, c);
+                        }
+                        wilson_hop_dir<double, double>(P.g, P.U64, P.antip, s, xc, mu, dir > 0, f, acc);
+                    }
+#pragma unroll
+                for (int c = 0; c < 12; ++c)
+                    bv[c] = cadd(source_val<1>(P, tk, key, s, xc, c), cscale(acc[c / 3][c % 3], kap));
+            }
+            if (plain_probe) {                     // units: |b|^2 counts them
+                const int32_t *col = P.col + (size_t)tk.cidx * P.g.N;
+                const int n = (col[s] == tk.colour) + (col[s ^ 1] == tk.colour);
+                v[1] += (double)(P.dilute ? n : 12 * n);
+            } else {
+                const int xp[4] = {xc[0] ^ 1, xc[1], xc[2], xc[3]};          // the odd site of the same entry
 #pragma unroll
                 for (int c = 0; c < 12; ++c) {
                     const Cx<double> be = source_val<1>(P, tk, key, s, xc, c);
                     const Cx<double> bo = source_val<1>(P, tk, key, s ^ 1, xp, c);
                     v[1] += be.re * be.re + be.im * be.im + bo.re * bo.re + bo.im * bo.im;
-                    rv[c] = bs[c / 3][c % 3];                           // x = 0
-                }
-            } else {
-                Cx<double> acc[4][3];
-                wilson_hop_fetch<double, double>(
-                    P.g, [&](int y, int, int, Cx<double> f[4][3]) { load_spinor<double, double>(t, N, y >> 1, f); },
-                    P.U64, P.antip, s, xc, acc);
-                if (P.clover) {
-                    // r = b' - A_ee x + kappa^2 D_eo t64
-                    Cx<double> xv[12];
-#pragma unroll
-                    for (int c = 0; c < 12; ++c) xv[c] = ld_cx<double, double>(x, N, c, idx);
-                    clover_mul(P.CL64, N, 0, idx, xv);
-#pragma unroll
-                    for (int c = 0; c < 12; ++c)
-                        rv[c] = csub(ld_cx<double, double>(bp, N, c, idx), csub(xv[c], cscale(acc[c / 3][c % 3], k2)));
-                } else {
-                    // r = b' - x + kappa^2 D_eo t64, component by component
-#pragma unroll
-                    for (int c = 0; c < 12; ++c) {
-                        const Cx<double> bc = ld_cx<double, double>(bp, N, c, idx);
-                        const Cx<double> xcc = ld_cx<double, double>(x, N, c, idx);
-                        rv[c] = csub(bc, csub(xcc, cscale(acc[c / 3][c % 3], k2)));
-                    }
                 }
             }
-            Cx<R> rs[12];
+            store_spinor<double, double>(bp, N, idx, bv);
+            weo_start_any(P, j, idx, bv, v);
+        SITE_LOOP_END
+        item_store<3>(P, j, b, v, sh);
+    ITEM_LOOP_END
+}
+
+// outer step, part 2, at the even entries: r64 = b'_e - S x64; r = (S) r64
+// starts the inner solve (p = r0 = r, e = 0).  Partials as above.
+__global__ void __launch_bounds__(PT_BLOCK, 2) k_weo_outer_residual(EP P) {
+    __shared__ double sh[32 * 3];
+    const int N = P.nsite;
+    const double k2 = P.kappa * P.kappa;
+    const int ku = fx_link_exp(P.fx_em);
+    ITEM_LOOP(LIST_OUTER)
+        if (P.slots[j].phase != PH_OUTER) continue;
+        const double *x = P.x64 + (size_t)j * P.L;
+        const FxField ft = fx_t64(P, j);
+        const double *bp = P.b64 + (size_t)j * P.L;
+        double v[3] = {0.0, 0.0, 0.0};
+        SITE_LOOP(1)
+            int xc[4];
+            const int s = half_site(P.g, 0, idx, xc);
+            FxC acc[4][3];
+            const int E = fx_hop(P.g, ft, P.Ufx, ku, P.antip, 0, s, xc, acc);
+            const double sc = k2 * fx_pow2(E);
+            Cx<double> rv[12];
+#pragma unroll
+            for (int c = 0; c < 12; ++c) rv[c] = ld_cx<double, double>(x, N, c, idx);
+            if (P.clover) clover_mul(P.CL64, N, 0, idx, rv);
 #pragma unroll
             for (int c = 0; c < 12; ++c) {
-                v[0] += rv[c].re * rv[c].re + rv[c].im * rv[c].im;
-                rs[c] = Cx<R>{rnd<S, R>((R)rv[c].re), rnd<S, R>((R)rv[c].im)};
-                v[2] += (double)rs[c].re * (double)rs[c].re + (double)rs[c].im * (double)rs[c].im;
+                const Cx<double> bc = ld_cx<double, double>(bp, N, c, idx);
+                const FxC a = acc[c / 3][c % 3];
+                rv[c] = Cx<double>{fma(sc, (double)a.re, bc.re - rv[c].re), fma(sc, (double)a.im, bc.im - rv[c].im)};
             }
-            store_spinor<S, R>(r, N, idx, rs);
-            store_spinor<S, R>(pv, N, idx, rs);
-            store_spinor<S, R>(r0, N, idx, rs);
-            Cx<R> zero[12];
-#pragma unroll
-            for (int c = 0; c < 12; ++c) zero[c] = Cx<R>{R(0), R(0)};
-            store_spinor<S, R>(e, N, idx, zero);
+            weo_start_any(P, j, idx, rv, v);
         SITE_LOOP_END
         item_store<3>(P, j, b, v, sh);
     ITEM_LOOP_END
@@ -2054,7 +2220,8 @@ __global__ void __launch_bounds__(PT_BLOCK) k_weo_outer_residual(EP P) {
 // task that converged at its first step, where x = 0); with the clover term
 // x_o = A_oo^{-1} b_o + kappa t64, t64 = A_oo^{-1} D_oe x_e
 __device__ __forceinline__ void weo_x_at(const EP &P, const Task &tk, uint64_t key, const double *x,
-                                         const double *t64, int y, const int xy[4], Cx<double> out[12]) {
+                                         const double *t64, const int *et, int y, const int xy[4],
+                                         Cx<double> out[12]) {
     const int N = P.nsite;
     Cx<double> f[4][3];
     if (((xy[0] + xy[1] + xy[2] + xy[3]) & 1) == 0) {
@@ -2063,13 +2230,16 @@ __device__ __forceinline__ void weo_x_at(const EP &P, const Task &tk, uint64_t k
         for (int c = 0; c < 12; ++c) out[c] = f[c / 3][c % 3];
         return;
     }
-    load_spinor<double, double>(t64, N, y >> 1, f);
+    const double sc = P.kappa * fx_pow2(et[y >> 1]);           // t64 is in fixed point
+    FxC q[4][3];
+    fx_load(reinterpret_cast<const longlong2 *>(t64), N, y >> 1, q);
     Cx<double> bo[12];
 #pragma unroll
     for (int c = 0; c < 12; ++c) bo[c] = source_val<1>(P, tk, key, y, xy, c);
     if (P.clover && source_may_be_nonzero(P, tk, y)) clover_mul(P.CL64, N, 1, y >> 1, bo);   // A_oo^{-1} b_o
 #pragma unroll
-    for (int c = 0; c < 12; ++c) out[c] = cadd(bo[c], cscale(f[c / 3][c % 3], P.kappa));
+    for (int c = 0; c < 12; ++c)
+        out[c] = Cx<double>{fma(sc, (double)q[c / 3][c % 3].re, bo[c].re), fma(sc, (double)q[c / 3][c % 3].im, bo[c].im)};
 }
 
 // the contraction (trace mode) or the copy-out (solve mode) for even-odd
@@ -2084,6 +2254,7 @@ __global__ void __launch_bounds__(PT_BLOCK) k_weo_contract(EP P) {
         const Task tk = P.tasks[st.task];
         const double *x = P.x64 + (size_t)j * P.L;
         const double *t64 = P.t64 + (size_t)j * P.L;
+        const int *et = P.fx_et + (size_t)j * N;
         const uint64_t key = (P.mode == MODE_SOLVE) ? 0 : pt_set_key(P.seed, tk.set);
         if (P.mode == MODE_SOLVE) {
             SITE_LOOP(1)
@@ -2092,7 +2263,7 @@ __global__ void __launch_bounds__(PT_BLOCK) k_weo_contract(EP P) {
                     int xs[4];
                     site_coords(P.g, sw, xs);
                     Cx<double> xv[12];
-                    weo_x_at(P, tk, key, x, t64, sw, xs, xv);
+                    weo_x_at(P, tk, key, x, t64, et, sw, xs, xv);
                     double *dst = P.X_user + ((size_t)tk.set * NF + sw) * 24;
                     for (int c = 0; c < 12; ++c) {
                         dst[2 * c] = xv[c].re;
@@ -2128,7 +2299,7 @@ __global__ void __launch_bounds__(PT_BLOCK) k_weo_contract(EP P) {
                     for (int nu = 0; nu < 4; ++nu) xy[nu] = xs[nu];
                     xy[P.mu] = cm;
                     Cx<double> xv[12];
-                    weo_x_at(P, tk, key, x, t64, y, xy, xv);
+                    weo_x_at(P, tk, key, x, t64, et, y, xy, xv);
                     for (int a = 0; a < 12; ++a) {
                         if (P.dilute && a != tk.comp) continue;
                         const Cx<double> z = P.dilute ? pt_noise(key, (uint64_t)sw, P.noise)
@@ -2212,8 +2383,8 @@ __device__ __forceinline__ void wilson_hop_staged(const Geom &g, const S *f, int
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
                     Cx<R> t = cmul(sU[2 * mu][3 * a][col], h[k][0]);
-                    t = cadd(t, cmul(sU[2 * mu][3 * a + 1][col], h[k][1]));
-                    t = cadd(t, cmul(sU[2 * mu][3 * a + 2][col], h[k][2]));
+                    t = cmac(t, sU[2 * mu][3 * a + 1][col], h[k][1]);
+                    t = cmac(t, sU[2 * mu][3 * a + 2][col], h[k][2]);
                     uh[k][a] = t;
                 }
             spin_accumulate<R>(mu, R(-1), eta, uh, acc);
@@ -2229,8 +2400,8 @@ __device__ __forceinline__ void wilson_hop_staged(const Geom &g, const S *f, int
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
                     Cx<R> t = cconjmul(sU[2 * mu + 1][a][col], h[k][0]);
-                    t = cadd(t, cconjmul(sU[2 * mu + 1][3 + a][col], h[k][1]));
-                    t = cadd(t, cconjmul(sU[2 * mu + 1][6 + a][col], h[k][2]));
+                    t = cconjmac(t, sU[2 * mu + 1][3 + a][col], h[k][1]);
+                    t = cconjmac(t, sU[2 * mu + 1][6 + a][col], h[k][2]);
                     uh[k][a] = t;
                 }
             spin_accumulate<R>(mu, R(1), eta, uh, acc);
@@ -2440,7 +2611,12 @@ static void enqueue_iteration(const EngineRun &E, cudaStream_t st, const cudaEve
     }
     k_fin_contract<<<W, 256, 0, s_con>>>(Pc);
     ev_rec(ev, 5, s_out);
-    k_outer_update<KIND, S><<<E.g_oupd, P.bs, 0, s_out>>>(Po);
+    if constexpr (KIND == 1) {
+        if (P.eo) k_weo_outer_update<S><<<E.g_oupd, P.bs, 0, s_out>>>(Po);
+        else k_outer_update<KIND, S><<<E.g_oupd, P.bs, 0, s_out>>>(Po);
+    } else {
+        k_outer_update<KIND, S><<<E.g_oupd, P.bs, 0, s_out>>>(Po);
+    }
     if (P.eo) {
         if constexpr (KIND == 0) {
             k_eo_outer_hop<<<E.g_ohop, P.bs, 0, s_out>>>(Po);
@@ -2448,7 +2624,7 @@ static void enqueue_iteration(const EngineRun &E, cudaStream_t st, const cudaEve
         } else {
             k_weo_outer_hop<<<E.g_ohop, P.bs, 0, s_out>>>(Po);
             k_weo_outer_bprime<<<E.g_obp, P.bs, 0, s_out>>>(Po);
-            k_weo_outer_residual<S><<<E.g_ores, P.bs, 0, s_out>>>(Po);
+            k_weo_outer_residual<<<E.g_ores, P.bs, 0, s_out>>>(Po);
         }
     } else {
         k_outer_residual<KIND, S><<<E.g_ores, P.bs, 0, s_out>>>(Po);
@@ -2609,7 +2785,7 @@ static int run_engine_t(const pt_op *op, EngineRequest &rq, pt_stats *stats) {
         // a lattice that a thread-block cluster can hold is solved on chip, unless the
         // caller's tuning shapes this engine's work items or graphs, or caps its launches
         if (default_shape(tn) && c->launch_limit == 0 && pt_lap_resident_fits(op, rq, eo)) {
-            LapResidentPlan plan = {eo, tn.delta, cycle_slack(rq.prec), engine_max_inner(rq.prec, rq.maxit)};
+            LapResidentPlan plan = {eo, tn.delta, engine_max_inner(rq.prec, rq.maxit)};
             return pt_lap_resident_run(op, rq, plan, stats);
         }
     }
@@ -2619,11 +2795,16 @@ static int run_engine_t(const pt_op *op, EngineRequest &rq, pt_stats *stats) {
     // e, r, p, v, s, t, r0 (+ the odd-site hop buffer); FP64: x (+ t64, + b'_e)
     const int nvec = KIND ? (eo ? 8 : 7) : (eo ? 6 : 5);
     const int nf64 = eo ? 3 : 1;
-    const size_t per_slot = (size_t)L * (nf64 * sizeof(double) + nvec * sizeof(S));
+    // even-odd Wilson: the exponents of the fixed-point x64 and t64
+    const size_t fx_slot = (KIND == 1 && eo) ? (size_t)nsite * 2 * sizeof(int) : 0;
+    const size_t per_slot = (size_t)L * (nf64 * sizeof(double) + nvec * sizeof(S)) + fx_slot;
     // even-odd Wilson: the inner kernels read a copy of their links in the
     // even-odd order (LinkLayout<LS>::CHUNKS chunks per site)
     const size_t ueo_bytes = (KIND == 1 && eo) ? (size_t)g.N * LinkLayout<LS>::CHUNKS * sizeof(typename LinkLayout<LS>::E) : 0;
-    const size_t budget = c->mem_budget > 2 * ueo_bytes ? c->mem_budget - ueo_bytes : c->mem_budget / 2;
+    // and the outer step one as fixed-point digits
+    const size_t ufx_bytes = (KIND == 1 && eo) ? (size_t)g.N * 36 * sizeof(int4) : 0;
+    const size_t ucp_bytes = ueo_bytes + ufx_bytes;
+    const size_t budget = c->mem_budget > 2 * ucp_bytes ? c->mem_budget - ucp_bytes : c->mem_budget / 2;
     int R = rq.R_force > 0 ? rq.R_force : (int)std::min<size_t>((size_t)rq.n_tasks, budget / per_slot);
     if (rq.R_force <= 0 && c->max_slots > 0) R = std::min(R, c->max_slots);
     if (R < 1) R = 1;
@@ -2657,6 +2838,10 @@ static int run_engine_t(const pt_op *op, EngineRequest &rq, pt_stats *stats) {
     size_t o_tstat = take((size_t)rq.n_tasks * sizeof(TaskStat));
     size_t o_tout = take((size_t)rq.n_tasks * std::max(rq.n_p, 1) * 2 * sizeof(double));
     size_t o_ueo = ueo_bytes ? take(ueo_bytes) : 0;
+    size_t o_ufx = ufx_bytes ? take(ufx_bytes) : 0;
+    size_t o_fxem = take(sizeof(int));
+    size_t o_fxe = fx_slot ? take((size_t)R * nsite * sizeof(int)) : 0;
+    size_t o_fxt = fx_slot ? take((size_t)R * nsite * sizeof(int)) : 0;
     void *ws;
     int rc = pt_workspace(c, off, &ws);
     if (rc) return rc;
@@ -2666,6 +2851,7 @@ static int run_engine_t(const pt_op *op, EngineRequest &rq, pt_stats *stats) {
     memset(&P, 0, sizeof(P));
     P.g = g;
     P.kind = KIND;
+    P.prec = rq.prec;
     P.nsb = nsb;
     P.bs = bs;
     P.spt = spt;
@@ -2756,6 +2942,17 @@ static int run_engine_t(const pt_op *op, EngineRequest &rq, pt_stats *stats) {
             k_links_eo<E><<<c->num_sms * 8, 256, 0, st>>>(g, LinkLayout<LS>::CHUNKS, (const E *)P.U, ueo);
             PT_CUDA(cudaGetLastError());
             P.U = ueo;
+            int *em = (int *)(base + o_fxem);
+            int4 *ufx = (int4 *)(base + o_ufx);
+            PT_CUDA(cudaMemsetAsync(em, 0, sizeof(int), st));
+            k_fx_links_max<<<c->num_sms * 4, 256, 0, st>>>((int64_t)g.N * 72, op->U64, em);
+            k_fx_links<true><<<c->num_sms * 8, 256, 0, st>>>(g, (const double2 *)op->U64, em, ufx);
+            pt_kernel_launch_count += 2;
+            PT_CUDA(cudaGetLastError());
+            P.fx_em = em;
+            P.Ufx = ufx;
+            P.fx_ex = (int *)(base + o_fxe);
+            P.fx_et = (int *)(base + o_fxt);
         }
     }
 
@@ -2792,7 +2989,8 @@ static int run_engine_t(const pt_op *op, EngineRequest &rq, pt_stats *stats) {
     } else if (eo) {
         E.g_contract = persistent_grid(k_weo_contract<16>, ns, bs);
         E.g_contract32 = persistent_grid(k_weo_contract<PT_MAX_P>, ns, bs);
-        E.g_ores = persistent_grid(k_weo_outer_residual<S>, ns, bs);
+        E.g_oupd = persistent_grid(k_weo_outer_update<S>, ns, bs);
+        E.g_ores = persistent_grid(k_weo_outer_residual, ns, bs);
         E.g_ohop = persistent_grid(k_weo_outer_hop, ns, bs);
         E.g_obp = persistent_grid(k_weo_outer_bprime, ns, bs);
         E.g_hop = clv ? persistent_grid(k_weo_hop<S, LS, 0, 1>, ns, bs) : persistent_grid(k_weo_hop<S, LS, 0>, ns, bs);

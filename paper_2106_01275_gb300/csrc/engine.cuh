@@ -58,19 +58,6 @@ __device__ __forceinline__ int shift_fwd(const Geom &g, int idx, const int x[4],
     return idx + (c - x[mu]) * g.stride[mu];
 }
 
-// |r|^2 at which an inner cycle that starts from the FP64 residual |r|^2 = rr
-// ends: a factor delta below its start, but the residual that the outer test
-// asks for (half of tol |b|) where that lies within `slack` (in |r|^2) of it.
-// Ending a little above the last target would buy one more FP64 residual and
-// one more restart for the few iterations between the two.
-__host__ __device__ __forceinline__ double cycle_target2(double delta, double slack, double tol, double b2, double rr) {
-    const double fin = 0.25 * tol * tol * b2, t = delta * delta * rr;
-    return t <= slack * fin ? fin : t;
-}
-// slack: FP32 storage carries a cycle a decade past the default delta of 1e-5
-// (the autotuner's usual choice is 1e-6); BF16 storage is at its limit at delta
-static inline double cycle_slack(int prec) { return prec == PT_PREC_MIXED_FP32 ? 100.0 : 4.0; }
-
 // CG keeps its search direction across an FP64 residual replacement (the
 // direction's weight is |r|^2 of the new residual over that of the last
 // iteration) as long as the new residual is the one the recursion had reached
@@ -81,7 +68,7 @@ static inline double cycle_slack(int prec) { return prec == PT_PREC_MIXED_FP32 ?
 // The inner tolerance and iteration bounds of a run, as run_engine_t sets them.
 struct LapResidentPlan {
     bool eo;                   // even Schur complement (every side even) or the full system
-    double delta, slack;
+    double delta;
     int max_inner;
 };
 

@@ -69,7 +69,7 @@ struct ResP {
     int *head, *flags;
     TaskStat *tstat;
     double *task_out;
-    double tol, delta, slack;
+    double tol, delta;
     int maxit, max_inner;
     long long max_steps;            // inner iterations + outer steps of one task before it gives up
 };
@@ -342,7 +342,7 @@ __device__ __forceinline__ void res_outer_step(const ResP &P, ResSh &sh, int ran
         sh.fresh = start || !(tot[2] <= PT_CG_KEEP * sh.rr_rec);
         res_scalar<R>(sh.beta) = (R)(sh.fresh ? 0.0 : tot[2] / sh.rr);
         sh.rr = tot[2];
-        sh.target2 = cycle_target2(P.delta, P.slack, P.tol, sh.b2, tot[2]);
+        sh.target2 = fmax(P.delta * P.delta * tot[2], 0.25 * P.tol * P.tol * sh.b2);
     }
 }
 
@@ -910,7 +910,6 @@ int pt_lap_resident_run(const pt_op *op, EngineRequest &rq, const LapResidentPla
     P.task_out = (double *)(b + o_out);
     P.tol = rq.tol;
     P.delta = plan.delta;
-    P.slack = plan.slack;
     P.maxit = rq.maxit;
     P.max_inner = plan.max_inner;
     P.max_steps = 2LL * rq.maxit + 400;

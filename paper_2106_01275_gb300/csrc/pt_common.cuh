@@ -113,6 +113,14 @@ template <typename R> __device__ __forceinline__ Cx<R> cmul(Cx<R> a, Cx<R> b) {
 template <typename R> __device__ __forceinline__ Cx<R> cconjmul(Cx<R> a, Cx<R> b) {  // conj(a) b
     return {a.re * b.re + a.im * b.im, a.re * b.im - a.im * b.re};
 }
+// t + a b and t + conj(a) b as one chain of fused multiply-adds (a product
+// added as a whole costs one more instruction per part)
+template <typename R> __device__ __forceinline__ Cx<R> cmac(Cx<R> t, Cx<R> a, Cx<R> b) {
+    return {fma(-a.im, b.im, fma(a.re, b.re, t.re)), fma(a.im, b.re, fma(a.re, b.im, t.im))};
+}
+template <typename R> __device__ __forceinline__ Cx<R> cconjmac(Cx<R> t, Cx<R> a, Cx<R> b) {
+    return {fma(a.im, b.im, fma(a.re, b.re, t.re)), fma(-a.im, b.re, fma(a.re, b.im, t.im))};
+}
 template <typename R> __device__ __forceinline__ Cx<R> ctimes_i(Cx<R> a) { return {-a.im, a.re}; }
 template <typename R> __device__ __forceinline__ Cx<R> cscale(Cx<R> a, R s) { return {a.re * s, a.im * s}; }
 
@@ -346,8 +354,8 @@ __device__ __forceinline__ void herm6_mul(const R w[36], Cx<R> v[6]) {
         for (int j = i + 1; j < 6; ++j) {
             const Cx<R> u = Cx<R>{w[k], w[k + 1]};
             k += 2;
-            o[i] = cadd(o[i], cmul(u, v[j]));
-            o[j] = cadd(o[j], cconjmul(u, v[i]));
+            o[i] = cmac(o[i], u, v[j]);
+            o[j] = cconjmac(o[j], u, v[i]);
         }
 #pragma unroll
     for (int i = 0; i < 6; ++i) v[i] = o[i];
@@ -411,8 +419,8 @@ __device__ __forceinline__ void wilson_hop_site(const Geom &g, const S *f, const
 #pragma unroll
                 for (int a = 0; a < 3; ++a) {
                     Cx<R> t = cmul(u[a][0], h[k][0]);
-                    t = cadd(t, cmul(u[a][1], h[k][1]));
-                    t = cadd(t, cmul(u[a][2], h[k][2]));
+                    t = cmac(t, u[a][1], h[k][1]);
+                    t = cmac(t, u[a][2], h[k][2]);
                     uh[k][a] = t;
                 }
             spin_accumulate<R>(mu, R(-1), eta, uh, acc);
@@ -431,8 +439,8 @@ __device__ __forceinline__ void wilson_hop_site(const Geom &g, const S *f, const
                 for (int a = 0; a < 3; ++a) {
                     // (U^dagger h)_a = sum_b conj(U_ba) h_b
                     Cx<R> t = cconjmul(u[0][a], h[k][0]);
-                    t = cadd(t, cconjmul(u[1][a], h[k][1]));
-                    t = cadd(t, cconjmul(u[2][a], h[k][2]));
+                    t = cconjmac(t, u[1][a], h[k][1]);
+                    t = cconjmac(t, u[2][a], h[k][2]);
                     uh[k][a] = t;
                 }
             spin_accumulate<R>(mu, R(1), eta, uh, acc);
@@ -470,8 +478,8 @@ __device__ __forceinline__ void wilson_hop_multi(const Geom &g, const S *const (
 #pragma unroll
                     for (int a = 0; a < 3; ++a) {
                         Cx<R> t = cmul(u[a][0], h[k][0]);
-                        t = cadd(t, cmul(u[a][1], h[k][1]));
-                        t = cadd(t, cmul(u[a][2], h[k][2]));
+                        t = cmac(t, u[a][1], h[k][1]);
+                        t = cmac(t, u[a][2], h[k][2]);
                         uh[k][a] = t;
                     }
                 spin_accumulate<R>(mu, R(-1), eta, uh, acc[n]);
@@ -492,8 +500,8 @@ __device__ __forceinline__ void wilson_hop_multi(const Geom &g, const S *const (
 #pragma unroll
                     for (int a = 0; a < 3; ++a) {
                         Cx<R> t = cconjmul(u[0][a], h[k][0]);
-                        t = cadd(t, cconjmul(u[1][a], h[k][1]));
-                        t = cadd(t, cconjmul(u[2][a], h[k][2]));
+                        t = cconjmac(t, u[1][a], h[k][1]);
+                        t = cconjmac(t, u[2][a], h[k][2]);
                         uh[k][a] = t;
                     }
                 spin_accumulate<R>(mu, R(1), eta, uh, acc[n]);
