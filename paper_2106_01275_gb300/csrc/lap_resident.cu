@@ -16,6 +16,8 @@
 // (twenty colourings, eight sets) 107.8 -> 46.4 ms; 9 x 7 x 11 x 15, full
 // system, 48 right-hand sides 4.02 -> 1.04 ms; 4^4, 12 right-hand sides
 // 880 -> 86 us; 16^4, 24 solves in FP64 4.20 -> 2.25 ms.
+// (Figures of the kernel as it was first taken; res_nbsum's loads have since
+// brought the four to 43.9 ms, 0.96 ms, 86 us and 2.21 ms.)
 //
 // What bounds it now: an iteration needs about 18 shared-memory wavefronts of
 // 128 bytes per 32 entries (two hops of 7.25, and p, t, e), 0.32 of the SMs'
@@ -221,23 +223,17 @@ __device__ __forceinline__ void res_nbsum(const ResP &P, const F *buf, const Res
                                           int nt_mine, int par, F acc[V]) {
     const F *own = buf + l;
     const uint32_t bit = 1u << u;
-    // the t neighbours first: at the slab's ends they are another CTA's, the longest way.
-    // t+: the next CTA's first plane past the slab's end; t-: the last plane of the one before
+    // The t neighbours first: at the slab's ends they are another CTA's, the
+    // longest way (t+: the next CTA's first plane, t-: the last plane of the one
+    // before).  Both are loaded through the cluster's address space wherever they
+    // lie: a branch around a remote load kept the loads of the next unit behind
+    // it (16^4: 46.4 ms with the branch, 43.9 without).
     F tf[V], tb[V], t[V];
-    if (!(n.th & bit)) {
-        res_ld<V>(own + P.st, tf);
-    } else {
-        const F *q = own - (nt_mine - 1) * P.st;
-        if (P.C == 1) res_ld<V>(q, tf);
-        else res_ldr<V>(q, rank + 1 == P.C ? 0 : rank + 1, tf);
-    }
-    if (!(n.tl & bit)) {
-        res_ld<V>(own - P.st, tb);
-    } else {
-        const int prev = rank == 0 ? P.C - 1 : rank - 1;
-        const F *q = own + ((prev == P.C - 1 ? P.nt_last : P.nt) - 1) * P.st;
-        if (P.C == 1) res_ld<V>(q, tb);
-        else res_ldr<V>(q, prev, tb);
+    {
+        const int prev = rank == 0 ? P.C - 1 : rank - 1, next = rank + 1 == P.C ? 0 : rank + 1;
+        const bool hi = (n.th & bit) != 0, lo = (n.tl & bit) != 0;
+        res_ldr<V>(own + (hi ? -(nt_mine - 1) * P.st : P.st), hi ? next : rank, tf);
+        res_ldr<V>(own + (lo ? ((prev == P.C - 1 ? P.nt_last : P.nt) - 1) * P.st : -P.st), lo ? prev : rank, tb);
     }
     if constexpr (EO) {
         const bool odd_x = ((n.par >> u) ^ (uint32_t)par) & 1u;
