@@ -65,9 +65,9 @@ struct EP {
     int clover;                // even-odd Wilson with a clover term: the packed chiral blocks below
     const float4 *CL32;        // 1 + C (even), (1 + C)^{-1} (odd) for FP32 / BF16 inner storage
     const double2 *CL64;       // the same in FP64 (and 1 + C on the odd sites)
-    const int4 *Ufx;           // even-odd Wilson: links as fixed-point digits (fixed.cuh), even-odd order
+    const int4 *Ufx;           // Wilson: links as fixed-point digits (fixed.cuh); even-odd order in even-odd mode
     const int *fx_em;          // and their exponent
-    int *fx_ex, *fx_et;        // exponents of the fixed-point x64 (even entries) and t64 (odd) [R][nsite]
+    int *fx_ex, *fx_et;        // exponents of the fixed-point x64 and (even-odd) t64 [R][nsite]
     int mode;
     const int32_t *col;
     uint64_t seed;
@@ -464,35 +464,26 @@ __global__ void k_fin_contract(EP P) {
 }
 
 // ------------------------------------------------------------------ outer (FP64) steps
-// x64 += e (FP64 defect-correction update); x64 = 0 for a newly started task
-template <int KIND, typename S>
+// Laplacian: x64 += e (FP64 defect-correction update); x64 = 0 for a newly started task
+template <typename S>
 __global__ void __launch_bounds__(PT_BLOCK) k_outer_update(EP P) {
-    typedef Fld<KIND, S> F;
     const int N = P.nsite;            // field entries per slot (N/2 in even-odd mode)
     ITEM_LOOP(LIST_OUTER)
         const int ph = P.slots[j].phase;
         if (ph != PH_START && ph != PH_OUTER) continue;
         double *x = P.x64 + (size_t)j * P.L;
         const S *e = slot_cptr<S>(P.e, j, P.L);
-        SITE_LOOP(KIND)
-            for (int c = 0; c < F::NC; ++c) {
-                Cx<double> v = {0.0, 0.0};
-                if (ph == PH_OUTER) {
-                    Cx<double> xv = Fld<KIND, double>::ld(x, N, c, idx);
-                    auto ev = F::ld(e, N, c, idx);
-                    v = Cx<double>{xv.re + (double)ev.re, xv.im + (double)ev.im};
-                }
-                Fld<KIND, double>::st(x, N, c, idx, v);
-            }
+        SITE_LOOP(0)
+            x[idx] = ph == PH_OUTER ? x[idx] + (double)ld_real(e, (size_t)idx) : 0.0;
         SITE_LOOP_END
     ITEM_LOOP_END
 }
 
-// r64 = b - A x64 in FP64; r = (S) r64 starts the inner solve (e = 0);
-// partials: |r64|^2, |b|^2, |r|^2 (of the rounded r)
-template <int KIND, typename S>
+// Laplacian: r64 = b - A x64 in FP64; r = (S) r64 starts the inner solve
+// (e = 0); partials: |r64|^2, |b|^2, |r|^2 (of the rounded r)
+template <typename S>
 __global__ void __launch_bounds__(PT_BLOCK) k_outer_residual(EP P) {
-    typedef Fld<KIND, S> F;
+    typedef Fld<0, S> F;
     typedef typename F::R R;
     __shared__ double sh[32 * 3];
     const int N = P.g.N;
@@ -503,34 +494,21 @@ __global__ void __launch_bounds__(PT_BLOCK) k_outer_residual(EP P) {
         const Task tk = P.tasks[st.task];
         const uint64_t key = (P.mode == MODE_SOLVE) ? 0 : pt_set_key(P.seed, tk.set);
         S *r = slot_ptr<S>(P.r, j, P.L);
-        S *pv = slot_ptr<S>(P.pv, j, P.L);
         S *e = slot_ptr<S>(P.e, j, P.L);
-        S *r0 = KIND ? slot_ptr<S>(P.r0, j, P.L) : nullptr;
         double v[3] = {0.0, 0.0, 0.0};
-        SITE_LOOP(KIND)
+        SITE_LOOP(0)
             int xc[4];
             site_coords(P.g, idx, xc);
-            Cx<double> ax[F::NC];
-            if (ph == PH_OUTER) {
-                apply_site<KIND, double, double, double>(P, P.x64 + (size_t)j * P.L, P.U64, idx, xc, ax);
-            } else {
-#pragma unroll
-                for (int c = 0; c < F::NC; ++c) ax[c] = Cx<double>{0.0, 0.0};
-            }
-            for (int c = 0; c < F::NC; ++c) {
-                Cx<double> bv = source_val<KIND>(P, tk, key, idx, xc, c);
-                Cx<double> rv = csub(bv, ax[c]);
-                v[0] += rv.re * rv.re + rv.im * rv.im;
-                v[1] += bv.re * bv.re + bv.im * bv.im;
-                Cx<R> rs = Cx<R>{rnd<S, R>((R)rv.re), rnd<S, R>((R)rv.im)};
-                F::st(r, N, c, idx, rs);
-                if constexpr (KIND == 1) {
-                    F::st(pv, N, c, idx, rs);
-                    F::st(r0, N, c, idx, rs);
-                }
-                F::st(e, N, c, idx, Cx<R>{R(0), R(0)});
-                v[2] += (double)rs.re * (double)rs.re + (double)rs.im * (double)rs.im;
-            }
+            double ax = 0.0;
+            if (ph == PH_OUTER) ax = lap_site<double, double>(P.g, P.x64 + (size_t)j * P.L, P.diag, idx, xc);
+            const double bv = source_val<0>(P, tk, key, idx, xc, 0).re;
+            const double rv = bv - ax;
+            v[0] += rv * rv;
+            v[1] += bv * bv;
+            const R rs = rnd<S, R>((R)rv);
+            st_real(r, (size_t)idx, rs);
+            st_real(e, (size_t)idx, R(0));
+            v[2] += (double)rs * (double)rs;
         SITE_LOOP_END
         item_store<3>(P, j, b, v, sh);
     ITEM_LOOP_END
@@ -1934,7 +1912,7 @@ __device__ __forceinline__ void fx_load(const longlong2 *q, int N, int h, FxC (&
 
 // x64 += e (x64 = 0 for a new task) and its fixed-point form
 template <typename S>
-__global__ void __launch_bounds__(PT_BLOCK) k_weo_outer_update(EP P) {
+__global__ void __launch_bounds__(PT_BLOCK) k_wil_outer_update(EP P) {
     typedef typename ArithT<S>::T R;
     const int N = P.nsite;
     ITEM_LOOP(LIST_OUTER)
@@ -1991,7 +1969,7 @@ __global__ void __launch_bounds__(PT_BLOCK, 2) k_weo_outer_hop(EP P) {
             } else {
                 int xc[4];
                 const int s = half_site(P.g, 1, idx, xc);
-                E = fx_hop(P.g, fx, P.Ufx, ku, P.antip, 1, s, xc, acc);
+                E = fx_hop<true>(P.g, fx, P.Ufx, ku, P.antip, 1, s, xc, acc);
                 if (P.clover) {
                     const double sc = fx_pow2(E);
                     Cx<double> v[12];
@@ -2196,7 +2174,7 @@ __global__ void __launch_bounds__(PT_BLOCK, 2) k_weo_outer_residual(EP P) {
             int xc[4];
             const int s = half_site(P.g, 0, idx, xc);
             FxC acc[4][3];
-            const int E = fx_hop(P.g, ft, P.Ufx, ku, P.antip, 0, s, xc, acc);
+            const int E = fx_hop<true>(P.g, ft, P.Ufx, ku, P.antip, 0, s, xc, acc);
             const double sc = k2 * fx_pow2(E);
             Cx<double> rv[12];
 #pragma unroll
@@ -2207,6 +2185,47 @@ __global__ void __launch_bounds__(PT_BLOCK, 2) k_weo_outer_residual(EP P) {
                 const Cx<double> bc = ld_cx<double, double>(bp, N, c, idx);
                 const FxC a = acc[c / 3][c % 3];
                 rv[c] = Cx<double>{fma(sc, (double)a.re, bc.re - rv[c].re), fma(sc, (double)a.im, bc.im - rv[c].im)};
+            }
+            weo_start_any(P, j, idx, rv, v);
+        SITE_LOOP_END
+        item_store<3>(P, j, b, v, sh);
+    ITEM_LOOP_END
+}
+
+// outer step on the full system: r64 = b - A x64 = b - x64 + kappa H x64 with
+// the hop in fixed point (9^3 x 20, 12 solves: 6.15 -> 5.52 ms) and b regenerated (= b for a new task); r = (S) r64
+// starts the inner solve.  Partials as above.
+__global__ void __launch_bounds__(PT_BLOCK, 2) k_wil_outer_residual(EP P) {
+    __shared__ double sh[32 * 3];
+    const int N = P.g.N;
+    const int ku = fx_link_exp(P.fx_em);
+    ITEM_LOOP(LIST_OUTER)
+        const Slot &st = P.slots[j];
+        const int ph = st.phase;
+        if (ph != PH_START && ph != PH_OUTER) continue;
+        const Task tk = P.tasks[st.task];
+        const uint64_t key = (P.mode == MODE_SOLVE) ? 0 : pt_set_key(P.seed, tk.set);
+        const FxField fx = fx_x64(P, j);
+        const double *x = P.x64 + (size_t)j * P.L;
+        double v[3] = {0.0, 0.0, 0.0};
+        SITE_LOOP(1)
+            int xc[4];
+            site_coords(P.g, idx, xc);
+            FxC acc[4][3];
+            double sc = 0.0;
+            if (ph == PH_OUTER) sc = P.kappa * fx_pow2(fx_hop<false>(P.g, fx, P.Ufx, ku, P.antip, 0, idx, xc, acc));
+            Cx<double> rv[12];
+#pragma unroll
+            for (int c = 0; c < 12; ++c) {
+                const Cx<double> bv = source_val<1>(P, tk, key, idx, xc, c);
+                rv[c] = bv;
+                if (ph == PH_START) {
+                    v[1] += bv.re * bv.re + bv.im * bv.im;
+                } else {
+                    const Cx<double> xv = ld_cx<double, double>(x, N, c, idx);
+                    const FxC a = acc[c / 3][c % 3];
+                    rv[c] = Cx<double>{fma(sc, (double)a.re, bv.re - xv.re), fma(sc, (double)a.im, bv.im - xv.im)};
+                }
             }
             weo_start_any(P, j, idx, rv, v);
         SITE_LOOP_END
@@ -2659,12 +2678,8 @@ static void enqueue_iteration(const EngineRun &E, cudaStream_t st, const cudaEve
     }
     k_fin_contract<<<W, 256, 0, s_con>>>(Pc);
     ev_rec(ev, 5, s_out);
-    if constexpr (KIND == 1) {
-        if (P.eo) k_weo_outer_update<S><<<E.g_oupd, P.bs, 0, s_out>>>(Po);
-        else k_outer_update<KIND, S><<<E.g_oupd, P.bs, 0, s_out>>>(Po);
-    } else {
-        k_outer_update<KIND, S><<<E.g_oupd, P.bs, 0, s_out>>>(Po);
-    }
+    if constexpr (KIND == 1) k_wil_outer_update<S><<<E.g_oupd, P.bs, 0, s_out>>>(Po);
+    else k_outer_update<S><<<E.g_oupd, P.bs, 0, s_out>>>(Po);
     if (P.eo) {
         if constexpr (KIND == 0) {
             k_eo_outer_hop<<<E.g_ohop, P.bs, 0, s_out>>>(Po);
@@ -2675,7 +2690,8 @@ static void enqueue_iteration(const EngineRun &E, cudaStream_t st, const cudaEve
             k_weo_outer_residual<<<E.g_ores, P.bs, 0, s_out>>>(Po);
         }
     } else {
-        k_outer_residual<KIND, S><<<E.g_ores, P.bs, 0, s_out>>>(Po);
+        if constexpr (KIND == 1) k_wil_outer_residual<<<E.g_ores, P.bs, 0, s_out>>>(Po);
+        else k_outer_residual<S><<<E.g_ores, P.bs, 0, s_out>>>(Po);
     }
     k_fin_outer<<<W, 256, 0, s_out>>>(Po);
     ev_rec(ev, 6, s_out);
@@ -2842,16 +2858,17 @@ static int run_engine_t(const pt_op *op, EngineRequest &rq, pt_stats *stats) {
     const int64_t L = eo ? (int64_t)nsite * (KIND ? 24 : 1) : pt_field_reals(op);
     // inner vectors: CG e, r, p (two buffers), q (+ t on the odd sites); BiCGStab
     // e, r, p, v, s, t, r0 (+ the odd-site hop buffer); FP64: x (+ t64, + b'_e)
-    const int nvec = KIND ? (eo ? 8 : 7) : (eo ? 6 : 5);
+    // (full-system Wilson in BF16 has an eighth, which only the outer step uses: see fx_x64)
+    const int nvec = KIND ? (eo || sizeof(S) == 2 ? 8 : 7) : (eo ? 6 : 5);
     const int nf64 = eo ? 3 : 1;
-    // even-odd Wilson: the exponents of the fixed-point x64 and t64
-    const size_t fx_slot = (KIND == 1 && eo) ? (size_t)nsite * 2 * sizeof(int) : 0;
+    // Wilson: the exponents of the fixed-point x64 and (even-odd) t64
+    const size_t fx_slot = KIND == 1 ? (size_t)nsite * (eo ? 2 : 1) * sizeof(int) : 0;
     const size_t per_slot = (size_t)L * (nf64 * sizeof(double) + nvec * sizeof(S)) + fx_slot;
     // even-odd Wilson: the inner kernels read a copy of their links in the
     // even-odd order (LinkLayout<LS>::CHUNKS chunks per site)
     const size_t ueo_bytes = (KIND == 1 && eo) ? (size_t)g.N * LinkLayout<LS>::CHUNKS * sizeof(typename LinkLayout<LS>::E) : 0;
-    // and the outer step one as fixed-point digits
-    const size_t ufx_bytes = (KIND == 1 && eo) ? (size_t)g.N * 36 * sizeof(int4) : 0;
+    // and the outer step (even-odd or not) one as fixed-point digits
+    const size_t ufx_bytes = KIND == 1 ? (size_t)g.N * 36 * sizeof(int4) : 0;
     const size_t ucp_bytes = ueo_bytes + ufx_bytes;
     const size_t budget = c->mem_budget > 2 * ucp_bytes ? c->mem_budget - ucp_bytes : c->mem_budget / 2;
     int R = rq.R_force > 0 ? rq.R_force : (int)std::min<size_t>((size_t)rq.n_tasks, budget / per_slot);
@@ -2890,7 +2907,7 @@ static int run_engine_t(const pt_op *op, EngineRequest &rq, pt_stats *stats) {
     size_t o_ufx = ufx_bytes ? take(ufx_bytes) : 0;
     size_t o_fxem = take(sizeof(int));
     size_t o_fxe = fx_slot ? take((size_t)R * nsite * sizeof(int)) : 0;
-    size_t o_fxt = fx_slot ? take((size_t)R * nsite * sizeof(int)) : 0;
+    size_t o_fxt = fx_slot && eo ? take((size_t)R * nsite * sizeof(int)) : 0;
     void *ws;
     int rc = pt_workspace(c, off, &ws);
     if (rc) return rc;
@@ -2991,18 +3008,19 @@ static int run_engine_t(const pt_op *op, EngineRequest &rq, pt_stats *stats) {
             k_links_eo<E><<<c->num_sms * 8, 256, 0, st>>>(g, LinkLayout<LS>::CHUNKS, (const E *)P.U, ueo);
             PT_CUDA(cudaGetLastError());
             P.U = ueo;
-            int *em = (int *)(base + o_fxem);
-            int4 *ufx = (int4 *)(base + o_ufx);
-            PT_CUDA(cudaMemsetAsync(em, 0, sizeof(int), st));
-            k_fx_links_max<<<c->num_sms * 4, 256, 0, st>>>((int64_t)g.N * 72, op->U64, em);
-            k_fx_links<true><<<c->num_sms * 8, 256, 0, st>>>(g, (const double2 *)op->U64, em, ufx);
-            pt_kernel_launch_count += 2;
-            PT_CUDA(cudaGetLastError());
-            P.fx_em = em;
-            P.Ufx = ufx;
-            P.fx_ex = (int *)(base + o_fxe);
-            P.fx_et = (int *)(base + o_fxt);
         }
+        int *em = (int *)(base + o_fxem);
+        int4 *ufx = (int4 *)(base + o_ufx);
+        PT_CUDA(cudaMemsetAsync(em, 0, sizeof(int), st));
+        k_fx_links_max<<<c->num_sms * 4, 256, 0, st>>>((int64_t)g.N * 72, op->U64, em);
+        if (eo) k_fx_links<true><<<c->num_sms * 8, 256, 0, st>>>(g, (const double2 *)op->U64, em, ufx);
+        else k_fx_links<false><<<c->num_sms * 8, 256, 0, st>>>(g, (const double2 *)op->U64, em, ufx);
+        pt_kernel_launch_count += 2;
+        PT_CUDA(cudaGetLastError());
+        P.fx_em = em;
+        P.Ufx = ufx;
+        P.fx_ex = (int *)(base + o_fxe);
+        P.fx_et = eo ? (int *)(base + o_fxt) : nullptr;
     }
 
     int occ = 0;
@@ -3016,8 +3034,13 @@ static int run_engine_t(const pt_op *op, EngineRequest &rq, pt_stats *stats) {
     const int ns = c->num_sms;
     E.g_contract = persistent_grid(k_contract<KIND, 16>, ns, bs);
     E.g_contract32 = persistent_grid(k_contract<KIND, PT_MAX_P>, ns, bs);
-    E.g_oupd = persistent_grid(k_outer_update<KIND, S>, ns, bs);
-    E.g_ores = persistent_grid(k_outer_residual<KIND, S>, ns, bs);
+    if constexpr (KIND == 1) {
+        E.g_oupd = persistent_grid(k_wil_outer_update<S>, ns, bs);
+        E.g_ores = persistent_grid(k_wil_outer_residual, ns, bs);
+    } else {
+        E.g_oupd = persistent_grid(k_outer_update<S>, ns, bs);
+        E.g_ores = persistent_grid(k_outer_residual<S>, ns, bs);
+    }
     E.g_hop = E.g_ohop = E.g_obp = 0;
     E.g_hop_g = E.g_apply1_g = E.g_apply2_g = 0;
     if constexpr (KIND == 0) {
@@ -3038,7 +3061,6 @@ static int run_engine_t(const pt_op *op, EngineRequest &rq, pt_stats *stats) {
     } else if (eo) {
         E.g_contract = persistent_grid(k_weo_contract<16>, ns, bs);
         E.g_contract32 = persistent_grid(k_weo_contract<PT_MAX_P>, ns, bs);
-        E.g_oupd = persistent_grid(k_weo_outer_update<S>, ns, bs);
         E.g_ores = persistent_grid(k_weo_outer_residual, ns, bs);
         E.g_ohop = persistent_grid(k_weo_outer_hop, ns, bs);
         E.g_obp = persistent_grid(k_weo_outer_bprime, ns, bs);

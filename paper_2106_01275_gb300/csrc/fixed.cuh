@@ -159,17 +159,20 @@ struct FxField {
     const int *e;
 };
 
-// (H psi)(x) at site idx of parity par: the integers in acc, the exponent
-// returned (FX_ZERO: all zero, FX_BAD: a NaN or infinity among the neighbours
-// or links).  f: half field (Nh entries) of the other parity; U: link digits
-// [4][9][N] in even-odd order, ku: their exponent.  The eight directions share
+// (H psi)(x) at site idx: the integers in acc, the exponent returned (FX_ZERO:
+// all zero, FX_BAD: a NaN or infinity among the neighbours or links).  EO: idx
+// has parity par, f is the half field of the other parity and U, the link
+// digits [4][9][N], are in even-odd order; else f is a full field and U by
+// site.  ku: the links' exponent.  The eight directions share
 // one copy of the products in a loop: unrolled, the 6400 instructions of a hop
 // were fetched from beyond the instruction cache (3.3 of 6.8 stall cycles per
 // instruction).
+template <bool EO>
 __device__ __forceinline__ int fx_hop(const Geom &g, const FxField &f, const int4 *U, int ku, int antip, int par,
                                       int idx, const int x[4], FxC (&acc)[4][3]) {
     const size_t N = (size_t)g.N;
-    const int Nh = g.N >> 1;
+    const int Ne = EO ? g.N >> 1 : g.N;
+    constexpr int half = EO ? 1 : 0;
 #pragma unroll
     for (int s = 0; s < 4; ++s)
 #pragma unroll
@@ -177,7 +180,8 @@ __device__ __forceinline__ int fx_hop(const Geom &g, const FxField &f, const int
     if (ku >= FX_BAD) return FX_BAD;         // a NaN or infinity among the links: so is every residual
     int E = FX_ZERO;
 #pragma unroll
-    for (int mu = 0; mu < 4; ++mu) E = max(E, max(f.e[nb_fwd(g, idx, x, mu) >> 1], f.e[nb_bwd(g, idx, x, mu) >> 1]));
+    for (int mu = 0; mu < 4; ++mu)
+        E = max(E, max(f.e[nb_fwd(g, idx, x, mu) >> half], f.e[nb_bwd(g, idx, x, mu) >> half]));
     if (E == FX_ZERO) return FX_ZERO;
 #pragma unroll 1
     for (int k = 0; k < 8; ++k) {
@@ -194,11 +198,11 @@ __device__ __forceinline__ int fx_hop(const Geom &g, const FxField &f, const int
             default: y = nb_bwd(g, idx, x, 3); neg = antip && x[3] == 0;
         }
         const bool bwd = k & 1;
-        const int yh = y >> 1;
+        const int yh = y >> half;
         FxC ps[4][3], h[2][3], uh[2][3];
 #pragma unroll
         for (int c = 0; c < 12; ++c) {
-            const longlong2 v = f.p[c / 3][(size_t)(c % 3) * Nh + yh];
+            const longlong2 v = f.p[c / 3][(size_t)(c % 3) * Ne + yh];
             ps[c / 3][c % 3] = FxC{v.x, v.y};
         }
         const int d = min(E - f.e[yh], 62);
@@ -221,7 +225,8 @@ __device__ __forceinline__ int fx_hop(const Geom &g, const FxField &f, const int
                 fx_digits(fx_down(h[q][a].im, d), hd[q][a].z, hd[q][a].w);
             }
         // U_mu(x) by rows, or the conjugate of U_mu(x - mu) by columns
-        const int4 *Uk = U + (size_t)(k >> 1) * 9 * N + (bwd ? (size_t)(1 - par) * Nh + yh : (size_t)par * Nh + (idx >> 1));
+        const int4 *Uk = U + (size_t)(k >> 1) * 9 * N + 
+                         (EO ? (bwd ? (size_t)(1 - par) * Ne + yh : (size_t)par * Ne + (idx >> 1)) : (size_t)(bwd ? y : idx));
         const size_t sa = (bwd ? 1 : 3) * N, sb = (bwd ? 3 : 1) * N;
         const int conj = bwd ? -1 : 0;
 #pragma unroll

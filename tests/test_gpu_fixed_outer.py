@@ -1,4 +1,4 @@
-"""The FP64 outer residual of the even-odd Wilson solve, whose hops run in
+"""The FP64 outer residual of the Wilson solve (even-odd and full system), whose hops run in
 block fixed point: solves to a tolerance near the FP64 floor, checked by the
 oracle's FP64 operator, where a wrong digit would show: unitary and scaled
 links, a point source (components over many orders of magnitude), a half
@@ -39,16 +39,19 @@ def _t(a):
     return torch.as_tensor(np.ascontiguousarray(a)).cuda()
 
 
-@pytest.mark.parametrize("dims,scale,csw", [([8, 8, 8, 16], 1.0, 0.0), ([6, 2, 4, 10], 1.0, 0.0), ([4, 6, 4, 8], 7.3, 0.0),
-                                            ([4, 4, 6, 8], 1.0, 1.1), ([2, 2, 2, 4], 0.01, 0.0)])
+@pytest.mark.parametrize("dims,scale,csw,eo", [([8, 8, 8, 16], 1.0, 0.0, 1), ([6, 2, 4, 10], 1.0, 0.0, 1),
+                                               ([4, 6, 4, 8], 7.3, 0.0, 1), ([4, 4, 6, 8], 1.0, 1.1, 1),
+                                               ([2, 2, 2, 4], 0.01, 0.0, 1), ([5, 3, 7, 9], 1.0, 0.0, 0),
+                                               ([1, 4, 2, 3], 2.5, 0.0, 0), ([4, 6, 4, 8], 1.0, 0.0, 0)])
 @pytest.mark.parametrize("prec", ["fp64", "mixed_fp32", "mixed_bf16"])
-def test_solve_near_the_fp64_floor(pt, ctx, dims, scale, csw, prec):
+def test_solve_near_the_fp64_floor(pt, ctx, dims, scale, csw, eo, prec):
     N = int(np.prod(dims))
     U = inputs.gauge_links(dims, 77) * scale
     kappa = 0.11 / scale
     op = pt.wilson(ctx, dims, _t(U), kappa, True)
     if csw:
         pt.set_clover(op, csw)
+    pt.set_tuning(op, prec, evenodd=eo)
     rng = np.random.default_rng(8)
     B = np.zeros((4, N, 4, 3), np.complex128)
     B[0, N // 3, 1, 2] = 1.0                                        # an even or odd point, and its neighbour
@@ -56,6 +59,7 @@ def test_solve_near_the_fp64_floor(pt, ctx, dims, scale, csw, prec):
     B[2] = rng.standard_normal((N, 4, 3)) + 1j * rng.standard_normal((N, 4, 3))
     B[3] = B[2] * 10.0 ** rng.uniform(-8, 0, (N, 1, 1))
     X, _, relres, _ = pt.solve(op, _t(B), prec, 1e-14, 20000)
+    pt.set_tuning(op, prec, reset=True)
     X = X.cpu().numpy()
     for j in range(4):
         ax = OC.clover_apply(X[j], U, kappa, csw, dims, True) if csw else OO.wilson_apply(X[j], U, kappa, dims, True)
