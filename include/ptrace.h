@@ -145,7 +145,8 @@ PT_API int pt_set_launch_limit(pt_ctx *ctx, int64_t n);
  *                S = 1 - kappa^2 D_eo D_oe, x_o = b_o + kappa D_oe x_e); the
  *                stopping test stays the full system's ||b - A x|| / ||b||.
  *                0: the full system.  The default is 1 where allowed; it is
- *                ignored for odd sides and by the Laplacian's pt_grad.
+ *                ignored for odd sides and by pt_grad, and it replaces
+ *                rhs_block by 1.
  *   cta_threads  threads of every work-item kernel's CTA: 64, 128 or 256
  *                (0 means 256)
  *   sites_per_thread  Laplacian: lattice sites (even-odd: half-lattice

@@ -2360,28 +2360,6 @@ __global__ void __launch_bounds__(PT_BLOCK) k_weo_contract(EP P) {
     ITEM_LOOP_END
 }
 
-// the whole solutions of a finished run, [slot][12][N] complex FP64 (the
-// gradient reads neighbours of both parities).  With them the gradient's
-// solves run on the even system, at half the iterations and half the vector
-// length: 8^3 x 16, 96 solves and the link outputs, 21.6 -> 10.4 ms.  Bound by
-// HBM: 384 bytes read and 384 written per entry
-__global__ void __launch_bounds__(128) k_weo_expand(EP P, double *out) {
-    const int NF = P.g.N, N = P.nsite;
-    const int64_t total = (int64_t)P.n_tasks * NF;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int j = (int)(i / NF), y = (int)(i - (int64_t)j * NF);
-        const Task tk = P.tasks[P.slots[j].task];
-        int x[4];
-        site_coords(P.g, y, x);
-        Cx<double> v[12];
-        weo_x_at(P, tk, pt_set_key(P.seed, tk.set), P.x64 + (size_t)j * P.L, P.t64 + (size_t)j * P.L,
-                 P.fx_et + (size_t)j * N, y, x, v);
-        double *f = out + (size_t)P.slots[j].task * 24 * NF;
-#pragma unroll
-        for (int c = 0; c < 12; ++c) st_cx<double, double>(f, NF, c, y, v[c]);
-    }
-}
-
 // ------------------------------------------------------------------ even-odd Wilson, link-sharing groups
 // rhs_block = 8 in even-odd mode: one CTA of 256 threads takes a block of 256
 // consecutive half-field entries for eight slots of the work list, one warp
@@ -2837,12 +2815,11 @@ static int run_engine_t(const pt_op *op, EngineRequest &rq, pt_stats *stats) {
     pt_ctx *c = op->ctx;
     const Geom g = op->g;
     const pt_ctx::Tune tn = engine_tuning(c, op, rq.prec);
-    // even-odd (every side even) unless switched off; the Laplacian's gradient
-    // works on full-lattice solutions and keeps the full system (Wilson: the
-    // solutions are expanded when the run is done)
+    // even-odd (every side even) unless switched off; the gradient works on
+    // full-lattice solutions and keeps the full system
     const bool clv = KIND == 1 && op->csw != 0.0;
-    const bool eo = (tn.evenodd || clv) && (KIND == 1 || rq.mode != MODE_GRAD) && pt_evenodd_ok(op->dims);
-    if (clv && (!eo || rq.mode == MODE_GRAD)) {
+    const bool eo = (tn.evenodd || clv) && rq.mode != MODE_GRAD && pt_evenodd_ok(op->dims);
+    if (clv && !eo) {
         pt_set_error("the clover operator runs on the even-odd engine only (every side even; no gradient)");
         return PT_ERR_ARG;
     }
@@ -3161,16 +3138,6 @@ static int run_engine_t(const pt_op *op, EngineRequest &rq, pt_stats *stats) {
     }
     PT_CUDA(cudaStreamSynchronize(st));
     rq.x64_out = P.x64;
-    if constexpr (KIND == 1) {
-        if (eo && rq.mode == MODE_GRAD) {
-            // into the inner vectors, which are free now and at least as large in every storage precision
-            double *full = (double *)(base + o_vec[0]);
-            k_weo_expand<<<c->num_sms * 8, 128, 0, st>>>(P, full);
-            ++pt_kernel_launch_count;
-            PT_CUDA(cudaGetLastError());
-            rq.x64_out = full;
-        }
-    }
     rq.R_used = R;
     if (stats) {
         memset(stats, 0, sizeof(*stats));
@@ -3498,37 +3465,29 @@ __global__ void k_grad_links(EP P, int n_pairs, double *G, double *Gb) {
     for (int i = 0; i < n_pairs; ++i) {
         const double *x = P.x64 + (size_t)(2 * i) * P.L;
         const double *w = P.x64 + (size_t)(2 * i + 1) * P.L;
-        // y^H (1 -+ g_mu) x = (half spinor of y)^H (half spinor of x): the projector is Hermitian and its square
-        // is twice itself, so two spins carry the product of four
-        Cx<double> hx[2][3], hy[2][3];
-        auto half = [&](const double *fld, int site, double sg, double g5, Cx<double>(&h)[2][3]) {
-            Cx<double> ps[4][3];
-            load_spinor<double, double>(fld, N, site, ps);
-#pragma unroll
-            for (int a = 0; a < 3; ++a) { ps[2][a] = cscale(ps[2][a], g5); ps[3][a] = cscale(ps[3][a], g5); }
-            switch (mu) {
-                case 0: spin_project<double>(0, sg, ps, h); break;
-                case 1: spin_project<double>(1, sg, ps, h); break;
-                case 2: spin_project<double>(2, sg, ps, h); break;
-                default: spin_project<double>(3, sg, ps, h);
+        Cx<double> ps[4][3], h[2][3], wv[4][3];
+        // (1 - g_mu) x(x + mu)
+        for (int s = 0; s < 4; ++s)
+            for (int a = 0; a < 3; ++a) { ps[s][a] = ld_cx<double, double>(x, N, 3 * s + a, f); wv[s][a] = Cx<double>{0, 0}; }
+        spin_project<double>(mu, -1.0, ps, h);
+        spin_accumulate<double>(mu, -1.0, 1.0, h, wv);
+        for (int s = 0; s < 4; ++s)
+            for (int a = 0; a < 3; ++a) {
+                Cx<double> y = ld_cx<double, double>(w, N, 3 * s + a, idx);
+                if (s >= 2) y = Cx<double>{-y.re, -y.im};
+                for (int bb = 0; bb < 3; ++bb) g[a][bb] = cadd(g[a][bb], cconjmul(y, wv[s][bb]));
             }
-        };
-        half(x, f, -1.0, 1.0, hx);            // (1 - g_mu) x(x + mu), y = g5 w at x
-        half(w, idx, -1.0, -1.0, hy);
-#pragma unroll
-        for (int k = 0; k < 2; ++k)
-#pragma unroll
-            for (int a = 0; a < 3; ++a)
-#pragma unroll
-                for (int bb = 0; bb < 3; ++bb) g[a][bb] = cconjmac(g[a][bb], hy[k][a], hx[k][bb]);
-        half(x, idx, 1.0, 1.0, hx);           // (1 + g_mu) x(x), y at x + mu
-        half(w, f, 1.0, -1.0, hy);
-#pragma unroll
-        for (int k = 0; k < 2; ++k)
-#pragma unroll
-            for (int a = 0; a < 3; ++a)
-#pragma unroll
-                for (int bb = 0; bb < 3; ++bb) gb[a][bb] = cconjmac(gb[a][bb], hy[k][bb], hx[k][a]);
+        // (1 + g_mu) x(x)
+        for (int s = 0; s < 4; ++s)
+            for (int a = 0; a < 3; ++a) { ps[s][a] = ld_cx<double, double>(x, N, 3 * s + a, idx); wv[s][a] = Cx<double>{0, 0}; }
+        spin_project<double>(mu, 1.0, ps, h);
+        spin_accumulate<double>(mu, 1.0, 1.0, h, wv);
+        for (int s = 0; s < 4; ++s)
+            for (int bb = 0; bb < 3; ++bb) {
+                Cx<double> y = ld_cx<double, double>(w, N, 3 * s + bb, f);
+                if (s >= 2) y = Cx<double>{-y.re, -y.im};
+                for (int a = 0; a < 3; ++a) gb[a][bb] = cadd(gb[a][bb], cconjmul(y, wv[s][a]));
+            }
     }
     const double kw = P.kappa * eta;
     double *go = G + ((size_t)idx * 4 + mu) * 18;
