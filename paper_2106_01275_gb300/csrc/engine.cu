@@ -3465,29 +3465,37 @@ __global__ void k_grad_links(EP P, int n_pairs, double *G, double *Gb) {
     for (int i = 0; i < n_pairs; ++i) {
         const double *x = P.x64 + (size_t)(2 * i) * P.L;
         const double *w = P.x64 + (size_t)(2 * i + 1) * P.L;
-        Cx<double> ps[4][3], h[2][3], wv[4][3];
-        // (1 - g_mu) x(x + mu)
-        for (int s = 0; s < 4; ++s)
-            for (int a = 0; a < 3; ++a) { ps[s][a] = ld_cx<double, double>(x, N, 3 * s + a, f); wv[s][a] = Cx<double>{0, 0}; }
-        spin_project<double>(mu, -1.0, ps, h);
-        spin_accumulate<double>(mu, -1.0, 1.0, h, wv);
-        for (int s = 0; s < 4; ++s)
-            for (int a = 0; a < 3; ++a) {
-                Cx<double> y = ld_cx<double, double>(w, N, 3 * s + a, idx);
-                if (s >= 2) y = Cx<double>{-y.re, -y.im};
-                for (int bb = 0; bb < 3; ++bb) g[a][bb] = cadd(g[a][bb], cconjmul(y, wv[s][bb]));
+        // y^H (1 -+ g_mu) x = (half spinor of y)^H (half spinor of x): the projector is Hermitian and its square
+        // is twice itself, so two spins carry the product of four
+        Cx<double> hx[2][3], hy[2][3];
+        auto half = [&](const double *fld, int site, double sg, double g5, Cx<double>(&h)[2][3]) {
+            Cx<double> ps[4][3];
+            load_spinor<double, double>(fld, N, site, ps);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) { ps[2][a] = cscale(ps[2][a], g5); ps[3][a] = cscale(ps[3][a], g5); }
+            switch (mu) {
+                case 0: spin_project<double>(0, sg, ps, h); break;
+                case 1: spin_project<double>(1, sg, ps, h); break;
+                case 2: spin_project<double>(2, sg, ps, h); break;
+                default: spin_project<double>(3, sg, ps, h);
             }
-        // (1 + g_mu) x(x)
-        for (int s = 0; s < 4; ++s)
-            for (int a = 0; a < 3; ++a) { ps[s][a] = ld_cx<double, double>(x, N, 3 * s + a, idx); wv[s][a] = Cx<double>{0, 0}; }
-        spin_project<double>(mu, 1.0, ps, h);
-        spin_accumulate<double>(mu, 1.0, 1.0, h, wv);
-        for (int s = 0; s < 4; ++s)
-            for (int bb = 0; bb < 3; ++bb) {
-                Cx<double> y = ld_cx<double, double>(w, N, 3 * s + bb, f);
-                if (s >= 2) y = Cx<double>{-y.re, -y.im};
-                for (int a = 0; a < 3; ++a) gb[a][bb] = cadd(gb[a][bb], cconjmul(y, wv[s][a]));
-            }
+        };
+        half(x, f, -1.0, 1.0, hx);            // (1 - g_mu) x(x + mu), y = g5 w at x
+        half(w, idx, -1.0, -1.0, hy);
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+#pragma unroll
+                for (int bb = 0; bb < 3; ++bb) g[a][bb] = cconjmac(g[a][bb], hy[k][a], hx[k][bb]);
+        half(x, idx, 1.0, 1.0, hx);           // (1 + g_mu) x(x), y at x + mu
+        half(w, f, 1.0, -1.0, hy);
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+#pragma unroll
+            for (int a = 0; a < 3; ++a)
+#pragma unroll
+                for (int bb = 0; bb < 3; ++bb) gb[a][bb] = cconjmac(gb[a][bb], hy[k][bb], hx[k][a]);
     }
     const double kw = P.kappa * eta;
     double *go = G + ((size_t)idx * 4 + mu) * 18;
