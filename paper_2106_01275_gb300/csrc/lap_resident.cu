@@ -89,6 +89,11 @@ struct ResSh {
     int cnt[RES_MAXW];
 };
 
+// the Z2 noise of a site as the sign bit of its hash (pt_noise without the FP64 pipe)
+__device__ __forceinline__ bool res_minus(uint64_t key, int site) {
+    return (pt_mix64(key + ((uint64_t)site + 1ULL) * PT_GAMMA) >> 63) != 0;
+}
+
 __device__ __forceinline__ uint32_t res_smem(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ uint32_t res_remote(const void *p, int rank) {
     uint32_t a;
@@ -408,7 +413,7 @@ __global__ void __launch_bounds__(TMAX, MINB) k_lap_resident(const __grid_consta
         const int32_t *col = P.mode == MODE_SOLVE ? nullptr : P.col + (size_t)tk.cidx * P.g.N;
         const double *bu = P.mode == MODE_SOLVE ? P.B_user + (size_t)tk.set * P.g.N : nullptr;
         auto probe_at = [&](int site) -> float {       // the probe's entry: 0 or +-1
-            return col[site] == tk.colour ? (float)pt_noise(key, (uint64_t)site, PT_NOISE_Z2).re : 0.f;
+            return col[site] == tk.colour ? (res_minus(key, site) ? -1.f : 1.f) : 0.f;
         };
 
         // -------- source: b' (x = 0, so r = b'), |b|^2, and the rounded r
@@ -474,7 +479,7 @@ __global__ void __launch_bounds__(TMAX, MINB) k_lap_resident(const __grid_consta
 #pragma unroll
                 for (int k = 0; k < V; ++k) {
                     zero[k] = 0.0;
-                    if (bp[k] != 0.0) v[0] += bp[k] * bp[k];   // a NaN is not equal to zero either
+                    v[0] += bp[k] * bp[k];
                     r[u][k] = res_rnd<S, R>((R)bp[k]);
                     v2 += r[u][k] * r[u][k];
                 }
@@ -630,7 +635,9 @@ __global__ void __launch_bounds__(TMAX, MINB) k_lap_resident(const __grid_consta
                 res_ld<V>(b64 + l, bp);
 #pragma unroll
                 for (int k = 0; k < V; ++k) {
-                    const double rv = EO ? bp[k] - (P.diag * x[k] - hs[k] * inv_dd) : bp[k] - (P.diag * x[k] - hs[k]);
+                    // b' - d x + H t / d, two fused multiply-adds
+                    const double rx = fma(-P.diag, x[k], bp[k]);
+                    const double rv = EO ? fma(hs[k], inv_dd, rx) : rx + hs[k];
                     v[0] += rv * rv;
                     r[u][k] = res_rnd<S, R>((R)rv);
                     v2 += r[u][k] * r[u][k];
@@ -685,7 +692,7 @@ __global__ void __launch_bounds__(TMAX, MINB) k_lap_resident(const __grid_consta
                 if (l < nv) in = P.n_lev ? P.lev_cols[site] == P.lev_anc[tk.colour] : col[site] == tk.colour;
                 const unsigned m = __ballot_sync(0xffffffffu, in);
                 if (in) {
-                    const bool neg = pt_noise(key, (uint64_t)site, PT_NOISE_Z2).re < 0.0;
+                    const bool neg = res_minus(key, site);
                     my[n_my + __popc(m & ((1u << lane) - 1u))] = site | (neg ? 1 << 30 : 0);
                 }
                 n_my += __popc(m);
@@ -768,9 +775,9 @@ static bool res_config(int elem, int V, int kbig, int ksmall, int tmax, const Ge
     int C = 1;
     while (C <= RES_MAXC && !(C <= Dt && fits(C))) C *= 2;
     if (C > RES_MAXC) return false;
-    // few right-hand sides: wider clusters use SMs that would stay idle, while
-    // a slab still has two units or more per thread of four warps
-    while (2 * C <= RES_MAXC && 2 * C <= Dt && (long)n_tasks * C * 2 <= num_sms && (Dt / (2 * C)) * st >= 256 * V) C *= 2;
+    // few right-hand sides: wider clusters use CTA slots (two per SM) that would
+    // stay idle, while a slab still has two units or more per thread of four warps
+    while (2 * C <= RES_MAXC && 2 * C <= Dt && (long)n_tasks * C <= num_sms && (Dt / (2 * C)) * st >= 256 * V) C *= 2;
     cf->nt = (Dt + C - 1) / C;
     cf->C = (Dt + cf->nt - 1) / cf->nt;                          // no CTA without a plane
     cf->nt_last = Dt - (cf->C - 1) * cf->nt;
