@@ -154,8 +154,9 @@ PT_API int pt_set_launch_limit(pt_ctx *ctx, int64_t n);
  *                a work item is cta_threads x sites_per_thread sites.  The
  *                Wilson kernels take one site per thread (pt_get_tuning
  *                reports 1).
- * A Laplacian lattice that a thread-block cluster can hold on chip (up to
- * 131,072 sites with even sides, 65,536 with odd ones, half of that in FP64) is solved by one
+ * A Laplacian lattice that a thread-block cluster of up to 16 CTAs can hold on
+ * chip (at most 262,144 sites with even sides, 131,072 with odd ones, half of
+ * that in FP64; less where the sides divide badly) is solved by one
  * kernel that keeps each right-hand side's vectors in shared memory and
  * registers, unless group, graph_iters, overlap, cta_threads or
  * sites_per_thread ask for a shape of the batched engine's work items other

@@ -2828,7 +2828,8 @@ static int run_engine_t(const pt_op *op, EngineRequest &rq, pt_stats *stats) {
         // caller's tuning shapes this engine's work items or graphs, or caps its launches
         if (default_shape(tn) && c->launch_limit == 0 && pt_lap_resident_fits(op, rq, eo)) {
             LapResidentPlan plan = {eo, tn.delta, engine_max_inner(rq.prec, rq.maxit)};
-            return pt_lap_resident_run(op, rq, plan, stats);
+            const int rres = pt_lap_resident_run(op, rq, plan, stats);
+            if (rres != PT_RES_NO_ROOM) return rres;
         }
     }
     const int nsite = eo ? g.N / 2 : g.N;

@@ -74,5 +74,7 @@ struct LapResidentPlan {
 
 // Whether a Laplacian run fits the cluster-resident solver (lap_resident.cu).
 bool pt_lap_resident_fits(const pt_op *op, const EngineRequest &rq, bool eo);
-// Runs it: fills rq.task_out, rq.tstat and *stats as the engine does.
+// Runs it: fills rq.task_out, rq.tstat and *stats as the engine does; PT_RES_NO_ROOM
+// (nothing done) where the device cannot schedule a cluster of the size needed.
+#define PT_RES_NO_ROOM 1
 int pt_lap_resident_run(const pt_op *op, EngineRequest &rq, const LapResidentPlan &plan, pt_stats *stats);

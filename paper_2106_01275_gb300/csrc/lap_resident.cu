@@ -44,7 +44,12 @@
 
 #include "engine.cuh"
 
-#define RES_MAXC 8                  // CTAs per cluster (the portable limit)
+// CTAs per cluster: above 8 by opt-in, only for lattices that 8 cannot hold
+// (measured against the batched engine, ms: 24 x 22 x 10 x 22, 64 solves 2.7 : 5.3;
+// 16^3 x 64, 64 solves 5.3 : 11.1; 16^2 x 24^2, 200 solves 7.7 : 14.4; 14 x 12 x 18^2
+// in FP64, 20 solves 2.4 : 4.6)
+#define RES_MAXC 16
+#define RES_PORTC 8                 // the portable limit
 #define RES_MAXW 16                 // warps per CTA
 
 struct ResP {
@@ -763,8 +768,8 @@ template <typename S> constexpr int res_minb(int V) { return 2; }
 constexpr int res_tmax(int V) { return V == 4 ? 256 : 512; }
 
 // CTAs per cluster, threads and build for n_tasks right-hand sides; false
-// where an xy plane exceeds a CTA's threads or eight CTAs cannot hold a slab
-// of t planes each
+// where an xy plane exceeds a CTA's threads or sixteen CTAs cannot hold a
+// slab of t planes each
 static bool res_config(int elem, int V, int kbig, int ksmall, int tmax, const Geom &g, int div, int n_tasks, int num_sms,
                        ResCfg *cf) {
     const int plane = g.D[0] / div * g.D[1] / V, st = g.stride[3] / div, Dt = g.D[3];
@@ -777,7 +782,7 @@ static bool res_config(int elem, int V, int kbig, int ksmall, int tmax, const Ge
     if (C > RES_MAXC) return false;
     // few right-hand sides: wider clusters use CTA slots (two per SM) that would
     // stay idle, while a slab still has two units or more per thread of four warps
-    while (2 * C <= RES_MAXC && 2 * C <= Dt && (long)n_tasks * C <= num_sms && (Dt / (2 * C)) * st >= 256 * V) C *= 2;
+    while (2 * C <= RES_PORTC && 2 * C <= Dt && (long)n_tasks * C <= num_sms && (Dt / (2 * C)) * st >= 256 * V) C *= 2;
     cf->nt = (Dt + C - 1) / C;
     cf->C = (Dt + cf->nt - 1) / cf->nt;                          // no CTA without a plane
     cf->nt_last = Dt - (cf->C - 1) * cf->nt;
@@ -843,7 +848,9 @@ int pt_lap_resident_run(const pt_op *op, EngineRequest &rq, const LapResidentPla
     lc.gridDim = dim3(cf.C);
     int n_cl = 0;
     if (cf.C > 1) {
+        if (cf.C > RES_PORTC) PT_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         PT_CUDA(cudaOccupancyMaxActiveClusters(&n_cl, kern, &lc));
+        if (n_cl < 1) return PT_RES_NO_ROOM;                     // (no GPC with that many free SMs)
     } else {
         PT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n_cl, kern, cf.T, cf.smem));
         n_cl *= c->num_sms;

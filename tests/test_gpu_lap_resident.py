@@ -1,5 +1,5 @@
 """The cluster-resident Laplacian solver against the batched engine and the
-oracle, over the forms that its dispatch accepts: one to eight CTAs per
+oracle, over the forms that its dispatch accepts: one to sixteen CTAs per
 cluster, slabs of unequal thickness, four-entry and one-entry units, even-odd
 and full system, every precision, solves, plain, nested and 32-output traces,
 and the caller's caps.  A tuning with its own graph length keeps the batched
@@ -38,19 +38,20 @@ def _t(a):
 # one CTA: a single site, sides of 1 and 2, a row of units; several: more t planes than CTAs, a last
 # slab of another thickness, one plane per CTA, planes that fill part of the threads
 SHAPES = [[1, 1, 1, 1], [3, 1, 5, 2], [2, 2, 2, 2], [8, 2, 2, 4], [6, 4, 2, 10], [16, 16, 16, 2], [8, 24, 6, 14],
-          [16, 16, 16, 16], [9, 13, 7, 11], [22, 23, 8, 9], [14, 18, 12, 18], [24, 22, 10, 22]]
+          [16, 16, 16, 16], [9, 13, 7, 11], [22, 23, 8, 9], [14, 18, 12, 18], [24, 22, 10, 22],
+          [26, 26, 6, 8], [8, 16, 16, 36]]
 
 
 def fits(dims, eo, prec):
     """The dispatch rule: the xy plane within a CTA's threads, and a slab of t
-    planes per CTA within its threads' entries for at most eight CTAs."""
+    planes per CTA within its threads' entries for at most sixteen CTAs."""
     v = 4 if eo and dims[0] % 8 == 0 else 1
     threads, entries = (256, 32) if v == 4 else (512, 16)
     entries //= 2 if prec == "fp64" else 1
     plane = dims[0] * dims[1] // (2 if eo else 1) // v
     if plane > threads:
         return False
-    return any(c <= dims[3] and -(-(-(-dims[3] // c) * dims[2]) // (threads // plane)) * v <= entries for c in (1, 2, 4, 8))
+    return any(c <= dims[3] and -(-(-(-dims[3] // c) * dims[2]) // (threads // plane)) * v <= entries for c in (1, 2, 4, 8, 16))
 
 
 @pytest.mark.parametrize("dims", SHAPES)
