@@ -240,6 +240,10 @@ def run_ours(args):
                  for k, v in (kv.split("=") for kv in args.tuning.split(","))}
         pt.set_tuning(op, args.prec, **fixed)
         tuning = pt.get_tuning(op, args.prec)
+    # Laplacian solves on chip touch a few MB of inputs: overwrite L2 before every step, inside the timed
+    # region (about 0.1 % of the step)
+    flush = (torch.empty(1 << 28, dtype=torch.uint8, device="cuda")
+             if W.kind == "lap" and torch.cuda.is_available() else None)
     for _ in range(args.warmup):
         step()
     torch.cuda.synchronize()
@@ -256,6 +260,8 @@ def run_ours(args):
     stats = []
     est = None
     for _ in range(args.steps):
+        if flush is not None:
+            flush.zero_()
         est, st = step()
         stats.append(st)
     ev1.record()
@@ -348,9 +354,11 @@ def run_ours(args):
                       "n_colours": m, "parallelism": "rhs-batched, %d rank(s), weak" % world,
                       "tuning": tuning,
                       "solver": ("even-odd (Schur complement on the even sites)" if eo else "full system"),
-                      "l2": "working set > L2 (resident RHS: %d, %.1f GB of inner vectors)" %
-                            (stats[-1]["n_slots"], stats[-1]["n_slots"] * vec_sites * n_vec *
-                             (4 if W.kind == "lap" else 96) / 1e9)},
+                      "l2": ("overwritten before every timed step (%d right-hand sides at a time, vectors held on "
+                             "chip)" % stats[-1]["n_slots"] if apply_launches == 0 and flush is not None else
+                             "working set > L2 (resident RHS: %d, %.1f GB of inner vectors)" %
+                             (stats[-1]["n_slots"], stats[-1]["n_slots"] * vec_sites * n_vec *
+                              (4 if W.kind == "lap" else 96) / 1e9))},
            "gpu_launches": int(launches), "roofline": roofline, "clocks": clocks,
            "mean_inner_iters_per_rhs": stats[-1]["inner_iters"] / stats[-1]["n_rhs"],
            "mean_outer_iters_per_rhs": stats[-1]["outer_iters"] / stats[-1]["n_rhs"],
