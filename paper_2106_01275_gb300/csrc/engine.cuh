@@ -62,8 +62,14 @@ __device__ __forceinline__ int shift_fwd(const Geom &g, int idx, const int x[4],
 // direction's weight is |r|^2 of the new residual over that of the last
 // iteration) as long as the new residual is the one the recursion had reached
 // (within half as much again); a fresh start would build up the Krylov space
-// anew at every cycle.
+// anew at every cycle.  At the same residual a solution reached that way has
+// more error left in the smooth modes than a restarted one (8^3 x 16, m^2 =
+// 0.16, displacement 5: 1.8e-9 of the estimate against 2.0e-10), so its last
+// cycle aims at an eighth of the tolerance: 1.9e-10 there, below the restarted
+// solves' error on every lattice tried, for one more iteration (16^4: 50.7
+// iterations a solve restarted, 46.7 kept, 48.9 kept and taken further).
 #define PT_CG_KEEP 2.25
+#define PT_CG_LAST2 0.015625
 
 // The inner tolerance and iteration bounds of a run, as run_engine_t sets them.
 struct LapResidentPlan {

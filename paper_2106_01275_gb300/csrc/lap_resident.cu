@@ -13,11 +13,9 @@
 // per right-hand side and iteration at 5.3 TB/s) and needs 12 launches per
 // iteration, which is all that small lattices spend their time on.  Measured
 // on one GB300, batched engine -> this kernel: 16^4, 4216 right-hand sides
-// (twenty colourings, eight sets) 107.8 -> 46.4 ms; 9 x 7 x 11 x 15, full
-// system, 48 right-hand sides 4.02 -> 1.04 ms; 4^4, 12 right-hand sides
-// 880 -> 86 us; 16^4, 24 solves in FP64 4.20 -> 2.25 ms.
-// (Figures of the kernel as it was first taken; res_nbsum's loads have since
-// brought the four to 43.9 ms, 0.96 ms, 86 us and 2.21 ms.)
+// (twenty colourings, eight sets) 107.8 -> 44.5 ms; 9 x 7 x 11 x 15, full
+// system, 48 right-hand sides 4.02 -> 0.96 ms; 4^4, 16 right-hand sides
+// 880 -> 86 us; 16^4, 24 solves in FP64 4.20 -> 2.20 ms.
 //
 // What bounds it now: an iteration needs about 18 shared-memory wavefronts of
 // 128 bytes per 32 entries (two hops of 7.25, and p, t, e), 0.32 of the SMs'
@@ -28,8 +26,8 @@
 // registers per SM, 32 entries per thread, four CTAs for 16^4.  Measured and
 // not taken at 16^4: eight CTAs of 16 entries per thread, three per SM,
 // 63 ms; two CTAs of 512 threads, one per SM, 49 ms.  The t neighbours that
-// lie in another CTA cost 1.6 ms of the 46.4 (with each slab closed on itself
-// instead: 44.8 ms).
+// lie in another CTA cost 1.6 ms of 46.4 (with each slab closed on itself
+// instead: 44.8 ms; before the last trims).
 //
 // The steps, the per-entry arithmetic and the order of its additions are the
 // engine's (k_eo_hop, k_eo_apply, k_cg_update, k_eo_outer_*, k_cg_apply,
@@ -349,6 +347,9 @@ __device__ __forceinline__ void res_outer_step(const ResP &P, ResSh &sh, int ran
         res_scalar<R>(sh.beta) = (R)(sh.fresh ? 0.0 : tot[2] / sh.rr);
         sh.rr = tot[2];
         sh.target2 = fmax(P.delta * P.delta * tot[2], 0.25 * P.tol * P.tol * sh.b2);
+        // a last cycle that keeps its direction goes on to an eighth of the tolerance (PT_CG_KEEP)
+        if (!sh.fresh && sh.target2 <= P.tol * P.tol * sh.b2)
+            sh.target2 = fmin(sh.target2, PT_CG_LAST2 * P.tol * P.tol * sh.b2);
     }
 }
 

@@ -106,3 +106,14 @@ def test_many_displacements_nested_levels_and_caps(pt, ctx):
     with pytest.raises(pt.PtraceError) as ei:
         pt.solve(op, _t(np.random.default_rng(1).standard_normal((3, N))), "mixed_fp32", 1e-12, 3)
     assert ei.value.code == pt.PT_ERR_NOCONV
+
+
+@pytest.mark.parametrize("dims,m2,mu,p", [([8, 8, 8, 16], 0.1587, 3, 5), ([12, 10, 10, 22], 0.1488, 0, 2)])
+def test_kept_direction_ends_below_the_tolerance(pt, ctx, dims, m2, mu, p):
+    """A last cycle that keeps its direction aims at tol / 8; it is kept only
+    where the FP64 residual is within 1.5 times the recursion's, so with FP32
+    drift of that size at most the final one is below 0.19 tol."""
+    col, m = pt.colour(ctx, dims, mu, [p], 1, "natural")
+    op = pt.laplacian(ctx, dims, m2)
+    _, _, _, st = pt.trace(op, col, m, mu, [p], "z2", 5, 0, 2, True, "mixed_fp32", 1e-10, 5000)
+    assert st["graph_launches"] == 0 and st["max_relres"] <= 0.19e-10
