@@ -727,7 +727,10 @@ static int colour_walk(pt_ctx *c, const int dims[4], int mu, const int *p_list, 
     size_t col_b = (size_t)g.N * sizeof(unsigned short);
     int max_smem = 0;
     PT_CUDA(cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, c->device));
-    max_smem -= 1024;  // static shared memory of the kernel
+    // less the static shared memory of the kernels.  Each kernel's limit is set to this and never to one
+    // call's own need: it belongs to the device, and contexts of other host threads launch the same kernels
+    // at other sizes in between.
+    max_smem -= 1024;
     PT_CHECK_ARG(stamp_b <= (size_t)max_smem, "pt_colour: stencil too large for the shared colour stamps");
     const bool sh_col = stamp_b + col_b <= (size_t)max_smem;
     const bool sh_off = stamp_b + off_b + (sh_col ? col_b : 0) <= (size_t)max_smem;
@@ -786,7 +789,7 @@ static int colour_walk(pt_ctx *c, const int dims[4], int mu, const int *p_list, 
 #define PT_WINDOW(T, NE)                                                                                         \
     do {                                                                                                         \
         PT_CUDA(cudaFuncSetAttribute(k_colour_window<T, false, NE>, cudaFuncAttributeMaxDynamicSharedMemorySize,  \
-                                     (int)smem));                                                                \
+                                     max_smem));                                                                 \
         k_colour_window<T, false, NE><<<1, 1024, smem, c->stream>>>(g, eg, wp, d_po, d_first, cp.d_visit, nullptr, \
                                                                     col_dev, cp.d_out, parent);                  \
     } while (0)
@@ -844,13 +847,13 @@ static int colour_walk(pt_ctx *c, const int dims[4], int mu, const int *p_list, 
 #define PT_EXT(U)                                                                                                \
     do {                                                                                                         \
         PT_CUDA(cudaFuncSetAttribute(k_colour_walk_ext<U>, cudaFuncAttributeMaxDynamicSharedMemorySize,          \
-                                     (int)ext_smem));                                                            \
+                                     max_smem));                                                                 \
         k_colour_walk_ext<U><<<1, PT_EXT_NT, ext_smem, c->stream>>>(g, eg, d_delta, n_off, cp.d_visit, d_ext,    \
                                                                     col_dev, n_stamp, cp.d_out);                 \
     } while (0)
         if (win_ext) {
             PT_CUDA(cudaFuncSetAttribute(k_colour_window<unsigned short, true, false>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)win_b));
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem));
             k_colour_window<unsigned short, true, false><<<1, 1024, win_b, c->stream>>>(
                 g, eg, wp, d_delta, d_first, cp.d_visit, d_ext, col_dev, cp.d_out, nullptr);
         }
@@ -874,7 +877,7 @@ static int colour_walk(pt_ctx *c, const int dims[4], int mu, const int *p_list, 
 #define PT_WALK(SC, SO, NE)                                                                                      \
     do {                                                                                                         \
         PT_CUDA(cudaFuncSetAttribute(k_colour_walk<SC, SO, NE>, cudaFuncAttributeMaxDynamicSharedMemorySize,      \
-                                     (int)shared_b));                                                            \
+                                     max_smem));                                                                 \
         k_colour_walk<SC, SO, NE><<<1, 1024, shared_b, c->stream>>>(g, d_off, n_off, cp.d_visit, col_dev,        \
                                                                     n_stamp, cp.d_out, parent);                  \
     } while (0)

@@ -813,6 +813,14 @@ bool pt_lap_resident_fits(const pt_op *op, const EngineRequest &rq, bool eo) {
 
 typedef void (*ResKernel)(const ResP);
 
+// Dynamic shared memory that a build may ask for: three arrays of its most
+// entries.  The kernel's limit is set to this, and never to one call's own
+// need: it belongs to the device, and contexts of other host threads launch
+// the same build at other sizes in between.
+static size_t res_smem_limit(int elem, int V, bool big, int kbig, int ksmall) {
+    return (size_t)3 * res_tmax(V) * (big ? kbig : ksmall) * elem;
+}
+
 template <typename S>
 static ResKernel res_kernel(bool eo, int V, bool big) {
     if (eo && V == 4)
@@ -834,7 +842,10 @@ int pt_lap_resident_run(const pt_op *op, EngineRequest &rq, const LapResidentPla
     ResKernel kern = rq.prec == PT_PREC_FP64 ? res_kernel<double>(plan.eo, V, cf.big)
                      : rq.prec == PT_PREC_MIXED_FP32 ? res_kernel<float>(plan.eo, V, cf.big)
                                                      : res_kernel<__nv_bfloat16>(plan.eo, V, cf.big);
-    PT_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cf.smem));
+    const size_t smem_limit = rq.prec == PT_PREC_FP64
+                                  ? res_smem_limit(8, V, cf.big, res_big<double>(V), res_small<double>(V))
+                                  : res_smem_limit(4, V, cf.big, res_big<float>(V), res_small<float>(V));
+    PT_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_limit));
     cudaLaunchConfig_t lc;
     memset(&lc, 0, sizeof(lc));
     cudaLaunchAttribute at[1];
