@@ -161,7 +161,9 @@ PT_API int pt_set_launch_limit(pt_ctx *ctx, int64_t n);
  * registers, unless group, graph_iters, overlap, cta_threads or
  * sites_per_thread ask for a shape of the batched engine's work items other
  * than the default, or a launch limit is set; pt_stats then counts one kernel
- * launch, no graph launches and the resident right-hand sides.
+ * launch, no graph launches and the resident right-hand sides.  On either path
+ * the bits of a solve or an estimate do not depend on how many others share
+ * its call.
  * seconds_per_rhs is an output of pt_autotune (device time per trial RHS). */
 typedef struct pt_tune {
     double delta;

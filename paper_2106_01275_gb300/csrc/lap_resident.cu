@@ -768,11 +768,9 @@ template <typename S> constexpr int res_small(int) { return 4; }
 template <typename S> constexpr int res_minb(int V) { return 2; }
 constexpr int res_tmax(int V) { return V == 4 ? 256 : 512; }
 
-// CTAs per cluster, threads and build for n_tasks right-hand sides; false
-// where an xy plane exceeds a CTA's threads or sixteen CTAs cannot hold a
-// slab of t planes each
-static bool res_config(int elem, int V, int kbig, int ksmall, int tmax, const Geom &g, int div, int n_tasks, int num_sms,
-                       ResCfg *cf) {
+// CTAs per cluster, threads and build; false where an xy plane exceeds a CTA's
+// threads or sixteen CTAs cannot hold a slab of t planes each
+static bool res_config(int elem, int V, int kbig, int ksmall, int tmax, const Geom &g, int div, ResCfg *cf) {
     const int plane = g.D[0] / div * g.D[1] / V, st = g.stride[3] / div, Dt = g.D[3];
     if (plane > tmax) return false;
     const int zs = tmax / plane;                                 // xy planes of units per step of the CTA
@@ -781,9 +779,12 @@ static bool res_config(int elem, int V, int kbig, int ksmall, int tmax, const Ge
     int C = 1;
     while (C <= RES_MAXC && !(C <= Dt && fits(C))) C *= 2;
     if (C > RES_MAXC) return false;
-    // few right-hand sides: wider clusters use CTA slots (two per SM) that would
-    // stay idle, while a slab still has two units or more per thread of four warps
-    while (2 * C <= RES_PORTC && 2 * C <= Dt && (long)n_tasks * C <= num_sms && (Dt / (2 * C)) * st >= 256 * V) C *= 2;
+    // The cluster depends on the lattice, the precision and the form, never on the
+    // number of right-hand sides: its CTAs fix the order in which a solve's sums
+    // are added, so that a solve has the same bits in a call of one as in a call of
+    // a thousand.  Wider clusters while CTA slots are free would speed up calls of
+    // a few solves (one on 9 x 7 x 11 x 15: 0.95 -> 0.52 ms, on 16^4 0.61 -> 0.47
+    // ms) and give nothing from 48 on (0.94 and 0.95 ms; 0.86 and 0.85 ms).
     cf->nt = (Dt + C - 1) / C;
     cf->C = (Dt + cf->nt - 1) / cf->nt;                          // no CTA without a plane
     cf->nt_last = Dt - (cf->C - 1) * cf->nt;
@@ -797,18 +798,18 @@ static bool res_config(int elem, int V, int kbig, int ksmall, int tmax, const Ge
     return steps(cf->nt, z) * V <= kpt;
 }
 
-static bool res_shape(const pt_op *op, const EngineRequest &rq, bool eo, int num_sms, int *V, ResCfg *cf) {
+static bool res_shape(const pt_op *op, const EngineRequest &rq, bool eo, int *V, ResCfg *cf) {
     const bool f64 = rq.prec == PT_PREC_FP64;
     *V = eo && op->g.D[0] % 8 == 0 ? 4 : 1;
     const int kb = f64 ? res_big<double>(*V) : res_big<float>(*V), ks = f64 ? res_small<double>(*V) : res_small<float>(*V);
-    return res_config(f64 ? 8 : 4, *V, kb, ks, res_tmax(*V), op->g, eo ? 2 : 1, rq.n_tasks, num_sms, cf);
+    return res_config(f64 ? 8 : 4, *V, kb, ks, res_tmax(*V), op->g, eo ? 2 : 1, cf);
 }
 
 bool pt_lap_resident_fits(const pt_op *op, const EngineRequest &rq, bool eo) {
     int V;
     ResCfg cf;
     return op->kind == 0 && rq.mode != MODE_GRAD && rq.R_force <= 0 && rq.n_tasks >= 1 &&
-           res_shape(op, rq, eo, op->ctx->num_sms, &V, &cf);
+           res_shape(op, rq, eo, &V, &cf);
 }
 
 typedef void (*ResKernel)(const ResP);
@@ -835,7 +836,7 @@ int pt_lap_resident_run(const pt_op *op, EngineRequest &rq, const LapResidentPla
     const Geom &g = op->g;
     int V;
     ResCfg cf;
-    if (!res_shape(op, rq, plan.eo, c->num_sms, &V, &cf)) {
+    if (!res_shape(op, rq, plan.eo, &V, &cf)) {
         pt_set_error("the lattice does not fit the resident solver");
         return PT_ERR_ARG;
     }
