@@ -65,8 +65,7 @@ struct EP {
     int clover;                // even-odd Wilson with a clover term: the packed chiral blocks below
     const float4 *CL32;        // 1 + C (even), (1 + C)^{-1} (odd) for FP32 / BF16 inner storage
     const double2 *CL64;       // the same in FP64 (and 1 + C on the odd sites)
-    const int4 *Ufx;           // Wilson: links as fixed-point digits (fixed.cuh); even-odd order in even-odd mode
-    const int *fx_em;          // and their exponent
+    FxLinks Ufx;               // Wilson: links in fixed point (fixed.cuh); even-odd order in even-odd mode
     int *fx_ex, *fx_et;        // exponents of the fixed-point x64 and (even-odd) t64 [R][nsite]
     int mode;
     const int32_t *col;
@@ -1954,7 +1953,6 @@ __global__ void __launch_bounds__(PT_BLOCK) k_wil_outer_update(EP P) {
 // hopped: the contraction reads it if the task converges at once)
 __global__ void __launch_bounds__(PT_BLOCK, 2) k_weo_outer_hop(EP P) {
     const int N = P.nsite;
-    const int ku = fx_link_exp(P.fx_em);
     ITEM_LOOP(LIST_OUTER)
         const int ph = P.slots[j].phase;
         if (ph != PH_START && ph != PH_OUTER) continue;
@@ -1969,7 +1967,7 @@ __global__ void __launch_bounds__(PT_BLOCK, 2) k_weo_outer_hop(EP P) {
             } else {
                 int xc[4];
                 const int s = half_site(P.g, 1, idx, xc);
-                E = fx_hop<true>(P.g, fx, P.Ufx, ku, P.antip, 1, s, xc, acc);
+                E = fx_hop<true>(P.g, fx, P.Ufx, P.antip, 1, s, xc, acc);
                 if (P.clover) {
                     const double sc = fx_pow2(E);
                     Cx<double> v[12];
@@ -2163,7 +2161,6 @@ __global__ void __launch_bounds__(PT_BLOCK, 2) k_weo_outer_residual(EP P) {
     __shared__ double sh[32 * 3];
     const int N = P.nsite;
     const double k2 = P.kappa * P.kappa;
-    const int ku = fx_link_exp(P.fx_em);
     ITEM_LOOP(LIST_OUTER)
         if (P.slots[j].phase != PH_OUTER) continue;
         const double *x = P.x64 + (size_t)j * P.L;
@@ -2174,7 +2171,7 @@ __global__ void __launch_bounds__(PT_BLOCK, 2) k_weo_outer_residual(EP P) {
             int xc[4];
             const int s = half_site(P.g, 0, idx, xc);
             FxC acc[4][3];
-            const int E = fx_hop<true>(P.g, ft, P.Ufx, ku, P.antip, 0, s, xc, acc);
+            const int E = fx_hop<true>(P.g, ft, P.Ufx, P.antip, 0, s, xc, acc);
             const double sc = k2 * fx_pow2(E);
             Cx<double> rv[12];
 #pragma unroll
@@ -2198,7 +2195,6 @@ __global__ void __launch_bounds__(PT_BLOCK, 2) k_weo_outer_residual(EP P) {
 __global__ void __launch_bounds__(PT_BLOCK, 2) k_wil_outer_residual(EP P) {
     __shared__ double sh[32 * 3];
     const int N = P.g.N;
-    const int ku = fx_link_exp(P.fx_em);
     ITEM_LOOP(LIST_OUTER)
         const Slot &st = P.slots[j];
         const int ph = st.phase;
@@ -2213,7 +2209,7 @@ __global__ void __launch_bounds__(PT_BLOCK, 2) k_wil_outer_residual(EP P) {
             site_coords(P.g, idx, xc);
             FxC acc[4][3];
             double sc = 0.0;
-            if (ph == PH_OUTER) sc = P.kappa * fx_pow2(fx_hop<false>(P.g, fx, P.Ufx, ku, P.antip, 0, idx, xc, acc));
+            if (ph == PH_OUTER) sc = P.kappa * fx_pow2(fx_hop<false>(P.g, fx, P.Ufx, P.antip, 0, idx, xc, acc));
             Cx<double> rv[12];
 #pragma unroll
             for (int c = 0; c < 12; ++c) {
@@ -2847,7 +2843,8 @@ static int run_engine_t(const pt_op *op, EngineRequest &rq, pt_stats *stats) {
     const size_t ueo_bytes = (KIND == 1 && eo) ? (size_t)g.N * LinkLayout<LS>::CHUNKS * sizeof(typename LinkLayout<LS>::E) : 0;
     // and the outer step (even-odd or not) one as fixed-point digits
     const size_t ufx_bytes = KIND == 1 ? (size_t)g.N * 36 * sizeof(int4) : 0;
-    const size_t ucp_bytes = ueo_bytes + ufx_bytes;
+    const size_t ufk_bytes = KIND == 1 ? (size_t)g.N * 4 * sizeof(int) : 0;
+    const size_t ucp_bytes = ueo_bytes + ufx_bytes + ufk_bytes;
     const size_t budget = c->mem_budget > 2 * ucp_bytes ? c->mem_budget - ucp_bytes : c->mem_budget / 2;
     int R = rq.R_force > 0 ? rq.R_force : (int)std::min<size_t>((size_t)rq.n_tasks, budget / per_slot);
     if (rq.R_force <= 0 && c->max_slots > 0) R = std::min(R, c->max_slots);
@@ -2883,7 +2880,7 @@ static int run_engine_t(const pt_op *op, EngineRequest &rq, pt_stats *stats) {
     size_t o_tout = take((size_t)rq.n_tasks * std::max(rq.n_p, 1) * 2 * sizeof(double));
     size_t o_ueo = ueo_bytes ? take(ueo_bytes) : 0;
     size_t o_ufx = ufx_bytes ? take(ufx_bytes) : 0;
-    size_t o_fxem = take(sizeof(int));
+    size_t o_ufk = ufk_bytes ? take(ufk_bytes) : 0;
     size_t o_fxe = fx_slot ? take((size_t)R * nsite * sizeof(int)) : 0;
     size_t o_fxt = fx_slot && eo ? take((size_t)R * nsite * sizeof(int)) : 0;
     void *ws;
@@ -2987,16 +2984,13 @@ static int run_engine_t(const pt_op *op, EngineRequest &rq, pt_stats *stats) {
             PT_CUDA(cudaGetLastError());
             P.U = ueo;
         }
-        int *em = (int *)(base + o_fxem);
         int4 *ufx = (int4 *)(base + o_ufx);
-        PT_CUDA(cudaMemsetAsync(em, 0, sizeof(int), st));
-        k_fx_links_max<<<c->num_sms * 4, 256, 0, st>>>((int64_t)g.N * 72, op->U64, em);
-        if (eo) k_fx_links<true><<<c->num_sms * 8, 256, 0, st>>>(g, (const double2 *)op->U64, em, ufx);
-        else k_fx_links<false><<<c->num_sms * 8, 256, 0, st>>>(g, (const double2 *)op->U64, em, ufx);
-        pt_kernel_launch_count += 2;
+        int *ufk = (int *)(base + o_ufk);
+        if (eo) k_fx_links<true><<<c->num_sms * 8, 256, 0, st>>>(g, (const double2 *)op->U64, ufx, ufk);
+        else k_fx_links<false><<<c->num_sms * 8, 256, 0, st>>>(g, (const double2 *)op->U64, ufx, ufk);
+        ++pt_kernel_launch_count;
         PT_CUDA(cudaGetLastError());
-        P.fx_em = em;
-        P.Ufx = ufx;
+        P.Ufx = FxLinks{ufx, ufk};
         P.fx_ex = (int *)(base + o_fxe);
         P.fx_et = eo ? (int *)(base + o_fxt) : nullptr;
     }

@@ -3,25 +3,34 @@
 // A GB300 SM issues two FP64 multiply-adds per cycle and 64 32-bit integer
 // ones, so the link products of the outer step run on the integer pipe:
 // a site's 12 complex components are 64-bit integers q with one exponent E
-// per site, value q 2^E, max |q| in [2^55, 2^56); a link entry is u = w 2^(k-57)
-// with |w| <= 2^57 and one k for the lattice.  Both are cut into two signed
+// per site, value q 2^E, |q| <= 2^56; a link entry is u = w 2^(k-57) with
+// |w| <= 2^57 and one k per link.  Both are cut into two signed
 // digits, q = q1 2^29 + q0 with q0 in [-2^28, 2^28), and
 //   (w q) 2^-57 = 2 w1 q1 + (w1 q0 + w0 q1) 2^-28 + w0 q0 2^-57
 // is summed exactly in two 64-bit accumulators (three 32 x 32 -> 64
 // multiply-adds per real product) but for the last term, below 1/2.
 //
-// Accuracy: a component within a factor 8 of its site's largest keeps all 53
-// bits of the double it came from; a smaller one is rounded at 2^-57 of the
-// largest.  Every hop sums components of neighbouring sites, so FP64
-// arithmetic rounds at 2^-53 of the largest partial sum as well; the total
-// error here is about a unit of 2^-56 of the largest neighbour component per
-// direction, below that of the FP64 hop it replaces.
+// Accuracy: converted from doubles, the largest |q| of a site and the largest
+// |w| of a link are at least 2^55 and 2^56, so a component within a factor 8 of
+// its site's largest keeps all 53 bits and a smaller one is rounded at 2^-57 of
+// the largest; an entry of a link within a factor 16 of the link's largest keeps
+// all its bits.  A hop adds its eight products at the exponent of the largest
+// (site exponent plus link exponent), about a unit of 2^-56 of that for each.
+// Its output (t64) keeps that exponent, also where the sum cancelled.  So errors
+// are small against the largest neighbour, not against each component: a result
+// far below its site's others has fewer right bits than in FP64 (1e-6 of them:
+// nine digits), and on links that leave the colours apart (U = 1) it has.
+// Where links mix them, FP64 rounds its sums at 2^-53 of the largest term too.
+// Errors against a 64-bit mantissa, root mean square over 8^3 x 16, kappa 0.12,
+// x the solution for one random source, FP64 hop -> this: links exp(0.3 i H) by
+// site norm 4.3e-17 -> 5.8e-18, by component 3.4e-16 -> 6.5e-17; U = 1 by site
+// norm 3.1e-17 -> 8.7e-18.
 #pragma once
 
 #include "pt_common.cuh"
 
 #define FX_ZERO (-(1 << 20))     // exponent of a site without a nonzero component
-#define FX_BAD (1 << 20)         // of a site (or link array) with a NaN or an infinity
+#define FX_BAD (1 << 22)         // of a site or link with a NaN or an infinity (FX_BAD + FX_ZERO is bad too)
 
 struct FxC { long long re, im; };
 
@@ -158,31 +167,39 @@ struct FxField {
     const longlong2 *p[4];
     const int *e;
 };
+// links: digits [4][9][N] and exponents [4][N], by site or in even-odd order
+struct FxLinks {
+    const int4 *u;
+    const int *k;
+};
 
 // (H psi)(x) at site idx: the integers in acc, the exponent returned (FX_ZERO:
 // all zero, FX_BAD: a NaN or infinity among the neighbours or links).  EO: idx
-// has parity par, f is the half field of the other parity and U, the link
-// digits [4][9][N], are in even-odd order; else f is a full field and U by
-// site.  ku: the links' exponent.  The eight directions share
-// one copy of the products in a loop: unrolled, the 6400 instructions of a hop
-// were fetched from beyond the instruction cache (3.3 of 6.8 stall cycles per
-// instruction).
+// has parity par, f is the half field of the other parity and the links are in
+// even-odd order; else f is a full field and the links by site.  The eight
+// directions share one copy of the products in a loop: unrolled, the 6400
+// instructions of a hop were fetched from beyond the instruction cache (3.3 of
+// 6.8 stall cycles per instruction).
 template <bool EO>
-__device__ __forceinline__ int fx_hop(const Geom &g, const FxField &f, const int4 *U, int ku, int antip, int par,
-                                      int idx, const int x[4], FxC (&acc)[4][3]) {
+__device__ __forceinline__ int fx_hop(const Geom &g, const FxField &f, const FxLinks &U, int antip, int par, int idx,
+                                      const int x[4], FxC (&acc)[4][3]) {
     const size_t N = (size_t)g.N;
     const int Ne = EO ? g.N >> 1 : g.N;
     constexpr int half = EO ? 1 : 0;
+    // entries of the links U_mu(x) and U_mu(y) in one of the nine arrays of a direction
+    const int own = EO ? par * Ne + (idx >> 1) : idx, other = EO ? (1 - par) * Ne : 0;
 #pragma unroll
     for (int s = 0; s < 4; ++s)
 #pragma unroll
         for (int a = 0; a < 3; ++a) acc[s][a] = FxC{0, 0};
-    if (ku >= FX_BAD) return FX_BAD;         // a NaN or infinity among the links: so is every residual
     int E = FX_ZERO;
 #pragma unroll
-    for (int mu = 0; mu < 4; ++mu)
-        E = max(E, max(f.e[nb_fwd(g, idx, x, mu) >> half], f.e[nb_bwd(g, idx, x, mu) >> half]));
-    if (E == FX_ZERO) return FX_ZERO;
+    for (int mu = 0; mu < 4; ++mu) {
+        const int yf = nb_fwd(g, idx, x, mu) >> half, yb = nb_bwd(g, idx, x, mu) >> half;
+        E = max(E, max(f.e[yf] + U.k[mu * N + own], f.e[yb] + U.k[mu * N + other + yb]));
+    }
+    if (E >= FX_BAD / 2) return FX_BAD;
+    if (E <= FX_ZERO / 2) return FX_ZERO;
 #pragma unroll 1
     for (int k = 0; k < 8; ++k) {
         int y;
@@ -205,7 +222,8 @@ __device__ __forceinline__ int fx_hop(const Geom &g, const FxField &f, const int
             const longlong2 v = f.p[c / 3][(size_t)(c % 3) * Ne + yh];
             ps[c / 3][c % 3] = FxC{v.x, v.y};
         }
-        const int d = min(E - f.e[yh], 62);
+        const int l = bwd ? other + yh : own;
+        const int d = min(E - f.e[yh] - U.k[(k >> 1) * N + l], 62);
         switch (k) {
             case 0: fx_project<0, -1>(ps, h); break;
             case 1: fx_project<0, 1>(ps, h); break;
@@ -225,8 +243,7 @@ __device__ __forceinline__ int fx_hop(const Geom &g, const FxField &f, const int
                 fx_digits(fx_down(h[q][a].im, d), hd[q][a].z, hd[q][a].w);
             }
         // U_mu(x) by rows, or the conjugate of U_mu(x - mu) by columns
-        const int4 *Uk = U + (size_t)(k >> 1) * 9 * N + 
-                         (EO ? (bwd ? (size_t)(1 - par) * Ne + yh : (size_t)par * Ne + (idx >> 1)) : (size_t)(bwd ? y : idx));
+        const int4 *Uk = U.u + (size_t)(k >> 1) * 9 * N + l;
         const size_t sa = (bwd ? 1 : 3) * N, sb = (bwd ? 3 : 1) * N;
         const int conj = bwd ? -1 : 0;
 #pragma unroll
@@ -251,7 +268,7 @@ __device__ __forceinline__ int fx_hop(const Geom &g, const FxField &f, const int
             default: fx_accumulate<3, 1>(uh, acc);
         }
     }
-    return E >= FX_BAD ? FX_BAD : E + ku;
+    return E;
 }
 
 // bring the integers below 2^56 again; returns the exponent that goes with them
@@ -275,34 +292,36 @@ __device__ __forceinline__ int fx_normalise(FxC (&q)[4][3], int E) {
     return E + d;
 }
 
-// ---- link digits: the largest exponent of the links, then the digits in the
-// even-odd link order (EO: chunk c of site s at c N + parity N/2 + s/2) or by site
-__global__ void k_fx_links_max(int64_t n, const double *__restrict__ U, int *em) {
-    int m = 1;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        m = max(m, (__double2hiint(U[i]) & 0x7fffffff) >> 20);
-    m = __reduce_max_sync(0xffffffffu, m);
-    if ((threadIdx.x & 31) == 0) atomicMax(em, m);
-}
-
+// ---- link digits and exponents, one thread per link: by site, or in the
+// even-odd link order (EO: site s of an array at parity N/2 + s/2)
 template <bool EO>
-__global__ void k_fx_links(Geom g, const double2 *__restrict__ src, const int *__restrict__ em_, int4 *__restrict__ dst) {
-    const int N = g.N, em = *em_;
-    const int64_t total = (int64_t)36 * N;
+__global__ void k_fx_links(Geom g, const double2 *__restrict__ src, int4 *__restrict__ dst, int *__restrict__ kexp) {
+    const int N = g.N;
+    const int64_t total = (int64_t)4 * N;
     for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t c = t / N;
-        const int s = (int)(t - c * N);
-        int64_t o = t;
+        const int64_t mu = t / N;
+        const int s = (int)(t - mu * N);
+        int o = s;
         if (EO) {
             int x[4];
             site_coords(g, s, x);
-            o = c * N + ((x[0] + x[1] + x[2] + x[3]) & 1) * (N >> 1) + (s >> 1);
+            o = ((x[0] + x[1] + x[2] + x[3]) & 1) * (N >> 1) + (s >> 1);
         }
-        const double2 v = src[t];
-        int4 d;
-        fx_digits(fx_quant(__double_as_longlong(v.x), em, 4), d.x, d.y);
-        fx_digits(fx_quant(__double_as_longlong(v.y), em, 4), d.z, d.w);
-        dst[o] = d;
+        double2 v[9];
+        int em = 1;
+#pragma unroll
+        for (int c = 0; c < 9; ++c) {
+            v[c] = src[(mu * 9 + c) * N + s];
+            em = max(em, (__double2hiint(v[c].x) & 0x7fffffff) >> 20);
+            em = max(em, (__double2hiint(v[c].y) & 0x7fffffff) >> 20);
+        }
+#pragma unroll
+        for (int c = 0; c < 9; ++c) {
+            int4 d;
+            fx_digits(fx_quant(__double_as_longlong(v[c].x), em, 4), d.x, d.y);
+            fx_digits(fx_quant(__double_as_longlong(v[c].y), em, 4), d.z, d.w);
+            dst[(mu * 9 + c) * N + o] = d;
+        }
+        kexp[mu * N + o] = em == 2047 ? FX_BAD : em - 1022;
     }
 }
-__device__ __forceinline__ int fx_link_exp(const int *em) { return *em >= 2047 ? FX_BAD : *em - 1022; }
