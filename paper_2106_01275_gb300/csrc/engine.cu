@@ -2045,21 +2045,19 @@ __device__ __forceinline__ void weo_probe_hop(const EP &P, const Task &tk, uint6
 // exact zeros), kept in FP64 for the task's later outer steps; x = 0, so
 // r64 = b'_e, and r = (S) r64 starts the inner solve (p = r0 = r, e = 0).
 // Partials: |r64|^2, |b|^2 of both sites of the entry (even and odd), |r|^2 of
-// the rounded r (summed per entry in the inner solve's arithmetic).
+// the rounded r, all in FP64: the last is the inner solve's rho and sets its target.
 template <typename S>
 __device__ __forceinline__ void weo_start_entry(const EP &P, int j, int idx, const Cx<double> (&rv)[12], double v[3]) {
     typedef typename ArithT<S>::T R;
     const int N = P.nsite;
     Cx<R> rs[12], zero[12];
-    R v2 = R(0);
 #pragma unroll
     for (int c = 0; c < 12; ++c) {
-        v[0] += rv[c].re * rv[c].re + rv[c].im * rv[c].im;
+        v[0] = fma(rv[c].im, rv[c].im, fma(rv[c].re, rv[c].re, v[0]));
         rs[c] = Cx<R>{rnd<S, R>((R)rv[c].re), rnd<S, R>((R)rv[c].im)};
-        v2 += rs[c].re * rs[c].re + rs[c].im * rs[c].im;
+        v[2] = fma((double)rs[c].im, (double)rs[c].im, fma((double)rs[c].re, (double)rs[c].re, v[2]));
         zero[c] = Cx<R>{R(0), R(0)};
     }
-    v[2] += (double)v2;
     store_spinor<S, R>(slot_ptr<S>(P.r, j, P.L), N, idx, rs);
     store_spinor<S, R>(slot_ptr<S>(P.pv, j, P.L), N, idx, rs);
     store_spinor<S, R>(slot_ptr<S>(P.r0, j, P.L), N, idx, rs);
