@@ -143,8 +143,8 @@ __device__ __forceinline__ void res_ldr(const double *p, int rank, double v[V]) 
 __device__ __forceinline__ void res_str(double *p, int rank, double v) {
     asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(res_remote(p, rank)), "d"(v) : "memory");
 }
-__device__ __forceinline__ void res_str(float *p, int rank, float v) {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(res_remote(p, rank)), "f"(v) : "memory");
+__device__ __forceinline__ void res_str(float2 *p, int rank, float2 v) {
+    asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(res_remote(p, rank)), "f"(v.x), "f"(v.y) : "memory");
 }
 __device__ __forceinline__ void res_str(int *p, int rank, int v) {
     asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(res_remote(p, rank)), "r"(v) : "memory");
@@ -281,14 +281,68 @@ __device__ __forceinline__ void res_nbsum(const ResP &P, const F *buf, const Res
     for (int k = 0; k < V; ++k) acc[k] += tb[k];
 }
 
+// Sums over a CTA's entries.  FP32 chains stay as short as the engine's, whose
+// warps add eight entries per lane and the 32 lanes in FP32: one sum per eight
+// entries of a thread (NG of them), each added over the warp by a tree of its
+// own; what is added beyond that is an unevaluated pair hi + lo (Knuth's
+// two-sum).  This and FP64 sums of |r|^2 on the full system against one FP32
+// chain over a thread's 16 or 32 entries: 16^4, 4216 solves 44.4 -> 45.6 ms;
+// 9 x 7 x 11 x 15, 48 solves 0.97 -> 1.02 ms.
+template <typename R, int KPT>
+struct ResAcc {
+    static constexpr int NG = std::is_same<R, float>::value && KPT > 8 ? KPT / 8 : 1;
+    R g[NG];
+    __device__ __forceinline__ ResAcc() {
+#pragma unroll
+        for (int i = 0; i < NG; ++i) g[i] = R(0);
+    }
+    // entry k of the thread (known where it is unrolled)
+    __device__ __forceinline__ void add(int k, R v) { g[NG == 1 ? 0 : k / 8] += v; }
+    __device__ __forceinline__ double total() const {
+        double s = (double)g[0];
+#pragma unroll
+        for (int i = 1; i < NG; ++i) s += (double)g[i];
+        return s;
+    }
+};
+
+__device__ __forceinline__ void res_pair(float &hi, float &lo, float h, float l) {
+    const float s = hi + h, b = s - hi;
+    lo = (lo + l) + ((hi - (s - b)) + (h - b));
+    hi = s;
+}
+__device__ __forceinline__ float res_xor(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+// half of the lanes go on with a, half with b, each taking the other half's
+__device__ __forceinline__ float res_split(float a, float b, int o) {
+    const bool h = (threadIdx.x & o) != 0;
+    return (h ? b : a) + res_xor(h ? a : b, o);
+}
+template <int KPT>
+__device__ __forceinline__ float2 res_warp(const ResAcc<float, KPT> &a) {
+    constexpr int NG = ResAcc<float, KPT>::NG;
+    static_assert(NG == 1 || NG == 2 || NG == 4, "sums of eight entries");
+    float hi, lo = 0.f;
+    if constexpr (NG == 4) hi = res_split(res_split(a.g[0], a.g[2], 16), res_split(a.g[1], a.g[3], 16), 8);
+    else if constexpr (NG == 2) hi = res_split(a.g[0], a.g[1], 16);
+    else hi = a.g[0];
+#pragma unroll
+    for (int o = 16 / NG; o > 0; o >>= 1) hi += res_xor(hi, o);
+    if constexpr (NG == 4) res_pair(hi, lo, res_xor(hi, 8), 0.f);
+    if constexpr (NG > 1) res_pair(hi, lo, res_xor(hi, 16), res_xor(lo, 16));
+    return make_float2(hi, lo);
+}
+
 template <typename R>
 __device__ __forceinline__ R &res_scalar(double &d) { return *reinterpret_cast<R *>(&d); }
 
-// Sums of K values over the cluster, in every lane of warp 0 of every CTA:
-// warp trees in T, the warp sums of all CTAs gathered in each, added in FP64
-// in a fixed order.  Contains one cluster barrier.
-template <int K, typename T>
-__device__ __forceinline__ void res_totals(ResSh &sh, int &buf, int C, int rank, T (&v)[K], double (&tot)[K]) {
+// shuffles that add up n values, one per lane or several, at lane 0
+__device__ __forceinline__ int res_span(int n) { return n > 16 ? 16 : n > 8 ? 8 : n > 4 ? 4 : n > 2 ? 2 : n > 1 ? 1 : 0; }
+
+// Sums of K FP64 values over the cluster, in thread 0 of every CTA (which alone
+// uses them: the upper lanes of its warp hold parts): warp trees, the warp sums
+// of all CTAs gathered in each, added in a fixed order.  One cluster barrier.
+template <int K>
+__device__ __forceinline__ void res_totals(ResSh &sh, int &buf, int C, int rank, double (&v)[K], double (&tot)[K]) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
     for (int k = 0; k < K; ++k)
@@ -297,10 +351,10 @@ __device__ __forceinline__ void res_totals(ResSh &sh, int &buf, int C, int rank,
     if (C == 1) {
         if (lane == 0)
 #pragma unroll
-            for (int k = 0; k < K; ++k) reinterpret_cast<T *>(sh.red[buf][k])[warp] = v[k];
+            for (int k = 0; k < K; ++k) sh.red[buf][k][warp] = v[k];
     } else if (lane < C) {
 #pragma unroll
-        for (int k = 0; k < K; ++k) res_str(reinterpret_cast<T *>(sh.red[buf][k]) + rank * nw + warp, lane, v[k]);
+        for (int k = 0; k < K; ++k) res_str(sh.red[buf][k] + rank * nw + warp, lane, v[k]);
     }
     res_sync(C);
     if (warp == 0) {
@@ -308,13 +362,44 @@ __device__ __forceinline__ void res_totals(ResSh &sh, int &buf, int C, int rank,
 #pragma unroll
         for (int k = 0; k < K; ++k) {
             double s = 0.0;
-            for (int i = lane; i < n; i += 32) s += (double)reinterpret_cast<const T *>(sh.red[buf][k])[i];
-            for (int o = (n > 16 ? 16 : n > 8 ? 8 : n > 4 ? 4 : n > 2 ? 2 : n > 1 ? 1 : 0); o > 0; o >>= 1)
-                s += __shfl_xor_sync(0xffffffffu, s, o);
+            for (int i = lane; i < n; i += 32) s += sh.red[buf][k][i];
+            for (int o = res_span(n); o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
             tot[k] = s;
         }
     }
     buf ^= 1;
+}
+
+// the same for one sum in the inner solve's arithmetic
+template <int KPT>
+__device__ __forceinline__ double res_total(ResSh &sh, int &buf, int C, int rank, const ResAcc<double, KPT> &a) {
+    double v[1] = {a.g[0]}, tot[1];
+    res_totals<1>(sh, buf, C, rank, v, tot);
+    return tot[0];
+}
+template <int KPT>
+__device__ __forceinline__ double res_total(ResSh &sh, int &buf, int C, int rank, const ResAcc<float, KPT> &a) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const float2 v = res_warp(a);
+    float2 *const red = reinterpret_cast<float2 *>(sh.red[buf][0]);
+    if (C == 1) {
+        if (lane == 0) red[warp] = v;
+    } else if (lane < C) {
+        res_str(red + rank * nw + warp, lane, v);
+    }
+    res_sync(C);
+    double s = 0.0;
+    if (warp == 0) {
+        const int n = C * nw;
+        for (int i = lane; i < n; i += 32) {
+            const float2 w = red[i];
+            s += (double)w.x;
+            if constexpr (ResAcc<float, KPT>::NG > 1) s += (double)w.y;
+        }
+        for (int o = res_span(n); o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    }
+    buf ^= 1;
+    return s;
 }
 
 // the engine's k_fin_outer (thread 0 of every CTA; CTA 0 reports)
@@ -425,7 +510,7 @@ __global__ void __launch_bounds__(TMAX, MINB) k_lap_resident(const __grid_consta
         // -------- source: b' (x = 0, so r = b'), |b|^2, and the rounded r
         {
             double v[3] = {0.0, 0.0, 0.0};
-            R v2 = R(0);
+            ResAcc<R, KPT> v2;
             if constexpr (EO) {
                 if (P.mode == MODE_SOLVE) {
                     RES_UNITS
@@ -487,16 +572,17 @@ __global__ void __launch_bounds__(TMAX, MINB) k_lap_resident(const __grid_consta
                     zero[k] = 0.0;
                     v[0] += bp[k] * bp[k];
                     r[u][k] = res_rnd<S, R>((R)bp[k]);
-                    v2 += r[u][k] * r[u][k];
+                    if constexpr (EO) v2.add(u * V + k, r[u][k] * r[u][k]);
+                    else v[2] += (double)r[u][k] * (double)r[u][k];
                 }
                 res_st<V>(b64 + l, bp);
                 res_st<V>(x64 + l, zero);
                 if constexpr (EO) res_st<V>(t64 + l, zero);
             RES_UNITS_END
             v[1] += (double)v1f;
-            v[2] = (double)v2;
+            v[2] += v2.total();
             double tot[3];
-            res_totals<3, double>(sh, buf, C, rank, v, tot);
+            res_totals<3>(sh, buf, C, rank, v, tot);
             if (tid == 0) res_outer_step<R>(P, sh, rank, true, tot);
             __syncthreads();
         }
@@ -542,7 +628,7 @@ __global__ void __launch_bounds__(TMAX, MINB) k_lap_resident(const __grid_consta
                     res_sync(C);
                 }
                 R q[U][V];
-                R pq[1] = {R(0)};
+                ResAcc<R, KPT> pq;
                 RES_UNITS
                     R hs[V], pc[V];
                     res_nbsum<EO, V, R>(P, EO ? ts : ps, nb, u, l, rank, nt_mine, 0, hs);
@@ -550,45 +636,44 @@ __global__ void __launch_bounds__(TMAX, MINB) k_lap_resident(const __grid_consta
 #pragma unroll
                     for (int k = 0; k < V; ++k) {
                         q[u][k] = res_rnd<S, R>(EO ? diag * pc[k] - hs[k] * inv_d : diag * pc[k] - hs[k]);
-                        pq[0] += pc[k] * q[u][k];
+                        pq.add(u * V + k, pc[k] * q[u][k]);
                     }
                 RES_UNITS_END
-                double tot[1];
-                res_totals<1, R>(sh, buf, C, rank, pq, tot);
+                double tot = res_total(sh, buf, C, rank, pq);
                 if (tid == 0) {
-                    if (!(tot[0] > 0.0) || !isfinite(tot[0])) {      // restart from the true residual
+                    if (!(tot > 0.0) || !isfinite(tot)) {            // restart from the true residual
                         if (rank == 0) atomicOr(&P.flags[FLAG_NUMERIC], 2);
                         sh.rr_rec = -1.0;
                         sh.phase = RS_OUTER;
                     } else {
-                        res_scalar<R>(sh.alpha) = (R)(sh.rr / tot[0]);
+                        res_scalar<R>(sh.alpha) = (R)(sh.rr / tot);
                     }
                 }
                 __syncthreads();
                 if (sh.phase == RS_OUTER) break;
                 al = res_scalar<R>(sh.alpha);
                 pending = true;
-                R rn[1] = {R(0)};
+                ResAcc<R, KPT> rn;
                 RES_UNITS
 #pragma unroll
                     for (int k = 0; k < V; ++k) {
                         r[u][k] = res_rnd<S, R>(r[u][k] - al * q[u][k]);
-                        rn[0] += r[u][k] * r[u][k];
+                        rn.add(u * V + k, r[u][k] * r[u][k]);
                     }
                 RES_UNITS_END
-                res_totals<1, R>(sh, buf, C, rank, rn, tot);
+                tot = res_total(sh, buf, C, rank, rn);
                 if (tid == 0) {
                     sh.inner_it += 1;
                     sh.total_it += 1;
                     sh.steps += 1;
-                    if (tot[0] <= sh.target2 || sh.inner_it >= P.max_inner || sh.total_it >= P.maxit ||
-                        !isfinite(tot[0]) || sh.steps >= P.max_steps) {
-                        sh.rr_rec = tot[0];
+                    if (tot <= sh.target2 || sh.inner_it >= P.max_inner || sh.total_it >= P.maxit ||
+                        !isfinite(tot) || sh.steps >= P.max_steps) {
+                        sh.rr_rec = tot;
                         sh.phase = RS_OUTER;
                     } else {
                         sh.fresh = 0;
-                        res_scalar<R>(sh.beta) = (R)(tot[0] / sh.rr);
-                        sh.rr = tot[0];
+                        res_scalar<R>(sh.beta) = (R)(tot / sh.rr);
+                        sh.rr = tot;
                     }
                 }
                 __syncthreads();
@@ -597,7 +682,7 @@ __global__ void __launch_bounds__(TMAX, MINB) k_lap_resident(const __grid_consta
 
             // -------- outer step: x64 += e, r = b' - S x64 (FP64), e = 0
             double v[3] = {0.0, 0.0, 0.0};
-            R v2 = R(0);
+            ResAcc<R, KPT> v2;
             // every read of p and t by another CTA is past a barrier of res_totals
             RES_UNITS
                 R e[V], pc[V];
@@ -646,13 +731,14 @@ __global__ void __launch_bounds__(TMAX, MINB) k_lap_resident(const __grid_consta
                     const double rv = EO ? fma(hs[k], inv_dd, rx) : rx + hs[k];
                     v[0] += rv * rv;
                     r[u][k] = res_rnd<S, R>((R)rv);
-                    v2 += r[u][k] * r[u][k];
+                    if constexpr (EO) v2.add(u * V + k, r[u][k] * r[u][k]);
+                    else v[2] += (double)r[u][k] * (double)r[u][k];
                 }
             RES_UNITS_END
             resume = true;
-            v[2] = (double)v2;
+            v[2] += v2.total();
             double tot[3];
-            res_totals<3, double>(sh, buf, C, rank, v, tot);
+            res_totals<3>(sh, buf, C, rank, v, tot);
             if (tid == 0) res_outer_step<R>(P, sh, rank, false, tot);
             __syncthreads();
         }
