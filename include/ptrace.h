@@ -105,7 +105,11 @@ PT_API int pt_destroy(pt_ctx *ctx);
 PT_API int pt_synchronize(pt_ctx *ctx);
 
 /* Cap on the device bytes the solver engine may hold for resident
- * right-hand sides (default 16 GiB).  Larger budgets keep more RHS in flight. */
+ * right-hand sides (default 16 GiB).  Larger budgets keep more RHS in flight.
+ * The Wilson engine's copies of the links count towards it: 592 bytes per site
+ * (fixed point, for the FP64 residual), and on the even-odd system one in the
+ * precision of the inner solve (144 to 576 bytes per site).  Whatever the cap,
+ * one right-hand side (pt_grad: one pair) and the copies are held. */
 PT_API int pt_set_memory_budget(pt_ctx *ctx, size_t bytes);
 
 /* Cap on the right-hand sides the solver engine keeps in flight (0 = no cap

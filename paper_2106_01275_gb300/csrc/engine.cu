@@ -2798,6 +2798,16 @@ static int engine_max_inner(int prec, int maxit) {
     return prec == PT_PREC_FP64 ? maxit : prec == PT_PREC_MIXED_FP32 ? 4000 : 400;
 }
 
+// Wilson: bytes of the links' fixed-point copy for the outer step (digits and exponents)
+static size_t fx_digit_bytes(const Geom &g) { return (size_t)g.N * 36 * sizeof(int4); }
+static size_t fx_link_bytes(const Geom &g) { return fx_digit_bytes(g) + (size_t)g.N * 4 * sizeof(int); }
+
+// What the context's memory budget leaves for right-hand sides beside the
+// engine's copies of the links (half of it where the copies would take more)
+static size_t slot_budget(const pt_ctx *c, size_t copies) {
+    return c->mem_budget > 2 * copies ? c->mem_budget - copies : c->mem_budget / 2;
+}
+
 // Laplacian: whether a tuning leaves the work items and graphs at their defaults
 static bool default_shape(const pt_ctx::Tune &t) {
     return t.group == 1 && t.graph_iters == 8 && t.overlap == 0 && (t.cta_threads == 0 || t.cta_threads == PT_BLOCK) &&
@@ -2840,10 +2850,9 @@ static int run_engine_t(const pt_op *op, EngineRequest &rq, pt_stats *stats) {
     // even-odd order (LinkLayout<LS>::CHUNKS chunks per site)
     const size_t ueo_bytes = (KIND == 1 && eo) ? (size_t)g.N * LinkLayout<LS>::CHUNKS * sizeof(typename LinkLayout<LS>::E) : 0;
     // and the outer step (even-odd or not) one as fixed-point digits
-    const size_t ufx_bytes = KIND == 1 ? (size_t)g.N * 36 * sizeof(int4) : 0;
-    const size_t ufk_bytes = KIND == 1 ? (size_t)g.N * 4 * sizeof(int) : 0;
-    const size_t ucp_bytes = ueo_bytes + ufx_bytes + ufk_bytes;
-    const size_t budget = c->mem_budget > 2 * ucp_bytes ? c->mem_budget - ucp_bytes : c->mem_budget / 2;
+    const size_t ufx_bytes = KIND == 1 ? fx_digit_bytes(g) : 0;
+    const size_t ufk_bytes = KIND == 1 ? fx_link_bytes(g) - ufx_bytes : 0;
+    const size_t budget = slot_budget(c, ueo_bytes + ufx_bytes + ufk_bytes);
     int R = rq.R_force > 0 ? rq.R_force : (int)std::min<size_t>((size_t)rq.n_tasks, budget / per_slot);
     if (rq.R_force <= 0 && c->max_slots > 0) R = std::min(R, c->max_slots);
     if (R < 1) R = 1;
@@ -3525,10 +3534,11 @@ extern "C" int pt_grad(pt_ctx *c, const pt_op *op, const int32_t *col_dev, int n
     std::vector<Task> all;
     build_probe_tasks(0, n_colours, set0, n_sets, op->dof, dilute, 1, all);
     const int n_pairs_total = (int)all.size() / 2;
-    // chunk of pairs resident at once
+    // chunk of pairs resident at once: x64, seven vectors and, for Wilson, the exponents of its fixed-point form
     const int64_t L = pt_field_reals(op);
-    const size_t per_slot = (size_t)L * (sizeof(double) + 7 * sizeof(double));
-    int Q = (int)std::max<size_t>(1, std::min<size_t>((size_t)n_pairs_total, c->mem_budget / (2 * per_slot)));
+    const size_t per_slot = (size_t)L * (sizeof(double) + 7 * sizeof(double)) + (op->kind == 1 ? (size_t)N * sizeof(int) : 0);
+    const size_t budget = slot_budget(c, op->kind == 1 ? fx_link_bytes(op->g) : 0);
+    int Q = (int)std::max<size_t>(1, std::min<size_t>((size_t)n_pairs_total, budget / (2 * per_slot)));
     Q = std::min(Q, 512);
     double dparam_re = 0.0, dparam_im = 0.0;
     std::vector<double> est(n_sets * 2, 0.0);
