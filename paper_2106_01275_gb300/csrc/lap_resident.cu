@@ -779,9 +779,12 @@ __global__ void __launch_bounds__(TMAX, MINB) k_lap_resident(const __grid_consta
             const int l = nb0.l0 + u * V * P.Te;
 #pragma unroll 1
             for (int k = 0; k < V * W2; ++k) {
-                const int site = W2 * (base + l) + k;
+                int site = 0;                        // (l of a thread without work is beyond what W2 l may be)
                 bool in = false;
-                if (l < nv) in = P.n_lev ? P.lev_cols[site] == P.lev_anc[tk.colour] : col[site] == tk.colour;
+                if (l < nv) {
+                    site = W2 * (base + l) + k;
+                    in = P.n_lev ? P.lev_cols[site] == P.lev_anc[tk.colour] : col[site] == tk.colour;
+                }
                 const unsigned m = __ballot_sync(0xffffffffu, in);
                 if (in) {
                     const bool neg = res_minus(key, site);
@@ -824,6 +827,7 @@ __global__ void __launch_bounds__(TMAX, MINB) k_lap_resident(const __grid_consta
             }
         }
         res_sync(C);
+        static_assert(PT_MAX_P <= 32, "one thread per output: a CTA has a warp at least");
         if (rank == 0 && tid < P.n_p) {
             double s = 0.0;
             for (int c = 0; c < C; ++c) s += sh.part[c][tid];
