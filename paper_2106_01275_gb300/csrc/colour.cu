@@ -857,8 +857,7 @@ static int colour_walk(pt_ctx *c, const int dims[4], int mu, const int *p_list, 
             k_colour_window<unsigned short, true, false><<<1, 1024, win_b, c->stream>>>(
                 g, eg, wp, d_delta, d_first, cp.d_visit, d_ext, col_dev, cp.d_out, nullptr);
         }
-        else if (n_off <= PT_EXT_NT * 4) PT_EXT(4);
-        else if (n_off <= PT_EXT_NT * 8) PT_EXT(8);
+        else if (n_off <= PT_EXT_NT * 8) PT_EXT(8);      // (the window takes stencils of up to about 5370 offsets)
         else if (n_off <= PT_EXT_NT * 12) PT_EXT(12);
         else if (n_off <= PT_EXT_NT * 16) PT_EXT(16);
         else if (n_off <= PT_EXT_NT * 20) PT_EXT(20);

@@ -113,23 +113,19 @@ __device__ __forceinline__ const T *slot_cptr(const void *base, int j, int64_t L
     return reinterpret_cast<const T *>(base) + (size_t)j * L;
 }
 
-// y = A f at one site (all NC components) in arithmetic R
-template <int KIND, typename R, typename S, typename LS>
+// Wilson: y = A f at one site in arithmetic R
+template <typename R, typename S, typename LS>
 __device__ __forceinline__ void apply_site(const EP &P, const S *f, const LS *U, int idx, const int x[4],
-                                           Cx<R> out[Fld<KIND, S>::NC]) {
-    if constexpr (KIND == 0) {
-        out[0] = Cx<R>{lap_site<R, S>(P.g, f, (R)P.diag, idx, x), R(0)};
-    } else {
-        Cx<R> acc[4][3];
-        wilson_hop_site<R, S, LS>(P.g, f, U, P.antip, idx, x, acc);
-        Cx<R> ps[4][3];
-        load_spinor<S, R>(f, P.g.N, idx, ps);
-        const R kap = (R)P.kappa;
+                                           Cx<R> out[12]) {
+    Cx<R> acc[4][3];
+    wilson_hop_site<R, S, LS>(P.g, f, U, P.antip, idx, x, acc);
+    Cx<R> ps[4][3];
+    load_spinor<S, R>(f, P.g.N, idx, ps);
+    const R kap = (R)P.kappa;
 #pragma unroll
-        for (int s = 0; s < 4; ++s)
+    for (int s = 0; s < 4; ++s)
 #pragma unroll
-            for (int a = 0; a < 3; ++a) out[3 * s + a] = csub(ps[s][a], cscale(acc[s][a], kap));
-    }
+        for (int a = 0; a < 3; ++a) out[3 * s + a] = csub(ps[s][a], cscale(acc[s][a], kap));
 }
 
 // source b(x, a) of a task
@@ -1238,7 +1234,7 @@ __global__ void __launch_bounds__(PT_BLOCK, std::is_same<S, double>::value ? 2 :
             int xc[4];
             site_coords(P.g, idx, xc);
             Cx<R> av[12];
-            apply_site<1, R, S, LS>(P, pv, (const LS *)P.U, idx, xc, av);
+            apply_site<R, S, LS>(P, pv, (const LS *)P.U, idx, xc, av);
             Cx<R> z[4][3];
             load_spinor<S, R>(r0, N, idx, z);
 #pragma unroll
@@ -1653,17 +1649,12 @@ __device__ __forceinline__ void wilson_hop_dir(const Geom &g, const LS *U, int a
 // that a warp of consecutive half entries reads consecutive links (in the
 // full-lattice order the sites of one parity are two apart)
 __device__ __forceinline__ int eo_link_pos(int N, int s, int par) { return par * (N >> 1) + (s >> 1); }
-template <int LPAR>
-__device__ __forceinline__ int link_pos(int N, int s, int par) {
-    if constexpr (LPAR < 0) return s;
-    else return eo_link_pos(N, s, par);
-}
 
 // (H psi)(x) at site idx (coordinates x) as in wilson_hop_site, with the
 // neighbour spinors supplied by fetch(y, mu, dir, ps) (dir +1 forward, -1
-// backward) and the links from a packed array in the full-lattice order
-// (LPAR = -1) or in the even-odd order with idx of parity LPAR
-template <typename R, typename LS, int LPAR = -1, typename Fetch>
+// backward) and the links from a packed array in the even-odd order; idx has
+// parity LPAR
+template <typename R, typename LS, int LPAR, typename Fetch>
 __device__ __forceinline__ void wilson_hop_fetch(const Geom &g, Fetch fetch, const LS *U, int antip, int idx,
                                                  const int x[4], Cx<R> acc[4][3]) {
 #pragma unroll
@@ -1679,7 +1670,7 @@ __device__ __forceinline__ void wilson_hop_fetch(const Geom &g, Fetch fetch, con
             Cx<R> ps[4][3], h[2][3], uh[2][3], u[3][3];
             fetch(y, mu, 1, ps);
             spin_project<R>(mu, R(-1), ps, h);
-            load_link<R, LS>(U, N, mu, link_pos<LPAR>(N, idx, LPAR), u);
+            load_link<R, LS>(U, N, mu, eo_link_pos(N, idx, LPAR), u);
 #pragma unroll
             for (int k = 0; k < 2; ++k)
 #pragma unroll
@@ -1697,7 +1688,7 @@ __device__ __forceinline__ void wilson_hop_fetch(const Geom &g, Fetch fetch, con
             Cx<R> ps[4][3], h[2][3], uh[2][3], u[3][3];
             fetch(y, mu, -1, ps);
             spin_project<R>(mu, R(1), ps, h);
-            load_link<R, LS>(U, N, mu, link_pos<LPAR>(N, y, 1 - LPAR), u);
+            load_link<R, LS>(U, N, mu, eo_link_pos(N, y, 1 - LPAR), u);
 #pragma unroll
             for (int k = 0; k < 2; ++k)
 #pragma unroll
