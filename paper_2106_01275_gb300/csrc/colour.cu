@@ -6,10 +6,11 @@
 // visit order.  What is parallel is the gather of the neighbourhood's colours
 // (Sec. 4 notes it is read-only): k_colour_window gathers for 31 nodes at once
 // while one warp settles the 31 before them in order.  Stencils whose stamps
-// do not fit 31 times in shared memory (beyond about 4700 offsets) are walked
-// one node at a time: k_colour_walk with the colours in shared or global
-// memory, k_colour_walk_ext with the colours in an extended array read through
-// L1 and two nodes in flight per barrier.
+// do not fit 31 times in shared memory (beyond about 5370 offsets; nested walks,
+// whose colours have to fit beside them, fewer) are walked one node at a time:
+// k_colour_walk with the colours in shared or global memory, k_colour_walk_ext
+// with the colours in an extended array read through L1 and two nodes in flight
+// per barrier.
 #include <limits.h>
 #include <string.h>
 
@@ -740,7 +741,7 @@ static int colour_walk(pt_ctx *c, const int dims[4], int mu, const int *p_list, 
     eg.k = k;
     eg.n_p = n_p;
     for (int n = 0; n < n_p; ++n) eg.p[n] = p_list[n] % dims[mu];
-    // the windowed walk wherever its stamps and rows (about 45 bytes per offset) fit: colours in shared
+    // the windowed walk wherever its stamps and rows (about 43 bytes per offset) fit: colours in shared
     // memory while they fit beside them, else in the extended array (not nested: its parents are by site)
     WinPar wp;
     memset(&wp, 0, sizeof(wp));

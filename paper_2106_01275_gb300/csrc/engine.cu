@@ -1863,7 +1863,9 @@ __global__ void __launch_bounds__(PT_BLOCK, weo_minb<S>(2 * CLV)) k_weo_apply2(E
 // the last subtraction and the sums are left on that pipe.  16^3 x 32, 48
 // right-hand sides, per outer step: hop 5.09 -> 1.76 ms, residual 6.04 -> 2.01 ms
 // (at 128 registers, 2 CTAs per SM, 0.5 KB of spills; without spills at one
-// CTA per SM 1.92 and 2.60 ms).  What bounds them: the integer pipes, each 64
+// CTA per SM 1.92 and 2.60 ms; before the links had an exponent each and |r|^2
+// was summed in FP64, which add 0.5 ms to the 57.5 ms of these solves with two
+// such steps each).  What bounds them: the integer pipes, each 64
 // lanes per SM and cycle (3400 multiply-adds and moves, 2900 additions, shifts
 // and selects per entry).
 //
@@ -2179,7 +2181,7 @@ __global__ void __launch_bounds__(PT_BLOCK, 2) k_weo_outer_residual(EP P) {
 }
 
 // outer step on the full system: r64 = b - A x64 = b - x64 + kappa H x64 with
-// the hop in fixed point (9^3 x 20, 12 solves: 6.15 -> 5.52 ms) and b regenerated (= b for a new task); r = (S) r64
+// the hop in fixed point (9^3 x 20, 12 solves: 6.15 -> 5.65 ms) and b regenerated (= b for a new task); r = (S) r64
 // starts the inner solve.  Partials as above.
 __global__ void __launch_bounds__(PT_BLOCK, 2) k_wil_outer_residual(EP P) {
     __shared__ double sh[32 * 3];

@@ -13,15 +13,15 @@
 // per right-hand side and iteration at 5.3 TB/s) and needs 12 launches per
 // iteration, which is all that small lattices spend their time on.  Measured
 // on one GB300, batched engine -> this kernel: 16^4, 4216 right-hand sides
-// (twenty colourings, eight sets) 107.8 -> 44.5 ms; 9 x 7 x 11 x 15, full
-// system, 48 right-hand sides 4.02 -> 0.96 ms; 4^4, 16 right-hand sides
-// 880 -> 86 us; 16^4, 24 solves in FP64 4.20 -> 2.20 ms.
+// (twenty colourings, eight sets) 107.8 -> 45.5 ms; 9 x 7 x 11 x 15, full
+// system, 48 right-hand sides 4.02 -> 1.00 ms; 4^4, 16 right-hand sides
+// 880 -> 86 us; 16^4, 24 solves in FP64 4.20 -> 2.21 ms.
 //
 // What bounds it now: an iteration needs about 18 shared-memory wavefronts of
-// 128 bytes per 32 entries (two hops of 7.25, and p, t, e), 0.32 of the SMs'
+// 128 bytes per 32 entries (two hops of 7.25, and p, t, e), 0.34 of the SMs'
 // shared-memory bandwidth at 16^4; the rest is latency (four cluster barriers
 // and two serial sums per iteration, 16 warps per SM to cover them and the
-// loads) and the FP64 pipe (0.38 busy: the outer steps' two hops).  So a
+// loads) and the FP64 pipe (0.28 busy: the outer steps' two hops).  So a
 // cluster is as small as its registers allow: two CTAs of 256 threads and 128
 // registers per SM, 32 entries per thread, four CTAs for 16^4.  Measured and
 // not taken at 16^4: eight CTAs of 16 entries per thread, three per SM,
@@ -29,11 +29,14 @@
 // lie in another CTA cost 1.6 ms of 46.4 (with each slab closed on itself
 // instead: 44.8 ms; before the last trims).
 //
-// The steps, the per-entry arithmetic and the order of its additions are the
-// engine's (k_eo_hop, k_eo_apply, k_cg_update, k_eo_outer_*, k_cg_apply,
-// k_outer_residual, k_contract): FP32 or BF16-rounded inner values with FP32
-// arithmetic inside FP64 defect correction, or FP64 throughout; dot products
-// as warp trees in the arithmetic type, then FP64 sums in a fixed order.
+// The steps and the per-entry arithmetic are the engine's (k_eo_hop, k_eo_apply,
+// k_cg_update, k_eo_outer_*, k_cg_apply, k_outer_residual, k_contract): FP32 or
+// BF16-rounded inner values with FP32 arithmetic inside FP64 defect correction,
+// or FP64 throughout; dot products as sums of eight entries and warp trees in
+// the arithmetic type, then FP64 sums in a fixed order.  Different on purpose:
+// CG keeps its direction across a residual replacement, and a last cycle that
+// kept it ends at an eighth of the tolerance (PT_CG_KEEP, PT_CG_LAST2); the
+// engine restarts and ends at the tolerance.
 #include <math.h>
 #include <stdio.h>
 #include <string.h>
